@@ -1,6 +1,5 @@
-// pa_gauss.cu — the Gaussian-coupling model (§II.A: J ~ N(0,1)): initial
-// energies, resampling from per-replica weights, energy moments and the link
-// overlap.  (Its sweep kernel, k_sweep_g, lives with the other sweep kernels.)
+// pa_gauss.cu — the Gaussian-coupling model (§II.A: J ~ N(0,1)):
+// resampling from per-replica weights, energy moments and the link overlap.  (Its sweep kernel, k_sweep_g, lives with the other sweep kernels.)
 //
 // Couplings and energies are fixed point (units of 2^-20, couplings clamped to
 // [-5, 5]), so energies, their sums and the link overlap are exact integers and
@@ -34,42 +33,9 @@ GArgs gpack(const PopDev* pops, int n_pop) {
 
 __host__ __device__ inline int blocks_for(long long n, int per) { return (int)((n + per - 1) / per); }
 
-constexpr uint32_t kBit1 = 0x02020202u;  // bit 1 of each byte: the two int8 spins differ
-
-// ---------------------------------------------------------------- initial energies
-
-// E_j = -sum_bonds J s s = -Jtot + 2 sum over antiparallel bonds of J, for the
-// four slots of one 32-bit word of every site row (int8 spins, site-major).
-__global__ void k_g_energy_init(RunGeom g, GArgs a, int cur, const int32_t* __restrict__ Jq) {
-  const PopDev& P = a.p[blockIdx.y];
-  const int R = P.rec[0].R_tilde;
-  const int wi = blockIdx.x * blockDim.x + threadIdx.x;
-  if (4 * wi >= R) return;
-  const int L = g.L;
-  const uint32_t* S = reinterpret_cast<const uint32_t*>(P.spins[cur]);
-  const int64_t pw = g.pitch / 4;
-  long long anti[4] = {0, 0, 0, 0}, jtot = 0;
-  for (int n = 0; n < g.N; ++n) {
-    const int x = n % L, y = (n / L) % L, z = n / (L * L);
-    const int nb[3] = {(x + 1 == L ? 0 : x + 1) + L * (y + L * z), x + L * ((y + 1 == L ? 0 : y + 1) + L * z),
-                       x + L * (y + L * (z + 1 == L ? 0 : z + 1))};
-    const uint32_t s = S[n * pw + wi];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const long long J = Jq[3 * n + d];
-      jtot += J;
-      const uint32_t x4 = (s ^ S[nb[d] * pw + wi]) & kBit1;
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if ((x4 >> (8 * b + 1)) & 1u) anti[b] += J;
-    }
-  }
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int j = 4 * wi + b;
-    if (j < R) P.E64[j] = -jtot + 2 * anti[b];
-  }
-}
+// Words of a warp's row in k_g_link: the sites, the first plane again, one word beyond
+// the last that a 32-bit read at any site's z neighbour touches.
+__host__ __device__ inline int link_row_words(int N, int L) { return (N + 31 + L * L) / 32 + 2; }
 
 // Opens the records of step t (what k_g_weights does for t >= 1).
 __global__ void k_g_open(GArgs a, int t) {
@@ -593,55 +559,95 @@ __global__ void __launch_bounds__(kMeasureThreads) k_g_count_E0(RunGeom g, GArgs
     atomicAdd(reinterpret_cast<unsigned long long*>(&P.grec[t].n_at_E0), (unsigned long long)c);
 }
 
-// Link overlap (Eq. ql) between slot j of the two populations, four pairs per
-// thread: with c = s1 s2 per site, QL = sum over bonds of c_n c_m = N_b - 2
-// (bonds whose c differ); histogram bin ((QL + N_b)(B - 1) + N_b) div 2N_b.
-__global__ void k_g_link(RunGeom g, GArgs a, int cur, int t, unsigned long long* qlhist) {
-  extern __shared__ unsigned int qh[];
+// Link overlap (Eq. ql) between slot j of the two populations: with c = s1 s2 per
+// site (the XOR of the two rows), QL = sum over bonds of c_n c_m = N_b - 2 (bonds
+// whose c differ); histogram bin ((QL + N_b)(B - 1) + N_b) div 2N_b.  One warp takes
+// a pair at a time: it holds the row c, padded with a copy of its first plane so that
+// the z neighbours of the last plane follow, in shared memory, and lane l counts the
+// bonds of the sites of words l, l + 32, ...: the neighbours of 32 consecutive sites
+// are 32 consecutive bits at an offset, but for the sites at the far edge of a row
+// (mask wx) or plane (mask wy), which take theirs from the row's or plane's start.
+// About 40 integer operations per 96 bonds; bound by HBM (two rows per pair).
+constexpr int kLinkThreads = 256;
+constexpr int kLinkPairsPerWarp = 16;
+
+// 32 bits of c from bit position pos on (pos >= 0, two words in range).
+__device__ __forceinline__ uint32_t bits_at(const uint32_t* c, int pos) {
+  return __funnelshift_r(c[pos >> 5], c[(pos >> 5) + 1], (uint32_t)pos & 31u);
+}
+
+__global__ void __launch_bounds__(kLinkThreads) k_g_link(RunGeom g, GArgs a, int cur, int t,
+                                                        unsigned long long* qlhist) {
+  extern __shared__ unsigned int qh[];  // [q_bins], masks wx and wy [nw each], then a padded row per warp
   __shared__ long long ssum;
   const PopDev& A = a.p[0];
   const PopDev& B = a.p[1];
   const int pairs = min(A.rec[t].R_tilde, B.rec[t].R_tilde);
+  const int L = g.L, N = g.N, nw = (N + 31) / 32, row_words = link_row_words(N, L);
+  uint32_t* wx = qh + g.q_bins;
+  uint32_t* wy = wx + nw;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t* c = wy + nw + warp * row_words;
   for (int i = threadIdx.x; i < g.q_bins; i += blockDim.x) qh[i] = 0u;
+  for (int k = threadIdx.x; k < nw; k += blockDim.x) {
+    uint32_t mx = 0, my = 0;
+    for (int b = 0; b < 32; ++b) {
+      const int n = 32 * k + b;
+      mx |= (uint32_t)(n % L == L - 1) << b;
+      my |= (uint32_t)((n / L) % L == L - 1) << b;
+    }
+    wx[k] = mx;
+    wy[k] = my;
+  }
   if (threadIdx.x == 0) ssum = 0;
   __syncthreads();
-  const int wi = blockIdx.x * blockDim.x + threadIdx.x;
-  const long long Nb = 3LL * g.N;
-  if (4 * wi < pairs) {
-    const int L = g.L;
-    const uint32_t* SA = reinterpret_cast<const uint32_t*>(A.spins[cur]);
-    const uint32_t* SB = reinterpret_cast<const uint32_t*>(B.spins[cur]);
-    const int64_t pw = g.pitch / 4;
-    int diff[4] = {0, 0, 0, 0};
-    uint32_t acc = 0;
-    int since = 0;
-    for (int n = 0; n < g.N; ++n) {
-      const int x = n % L, y = (n / L) % L, z = n / (L * L);
-      const int nx = (x + 1 == L ? 0 : x + 1) + L * (y + L * z);
-      const int ny = x + L * ((y + 1 == L ? 0 : y + 1) + L * z);
-      const int nz = x + L * (y + L * (z + 1 == L ? 0 : z + 1));
-      const uint32_t c = SA[n * pw + wi] ^ SB[n * pw + wi];
-      acc += ((c ^ SA[nx * pw + wi] ^ SB[nx * pw + wi]) & kBit1) + ((c ^ SA[ny * pw + wi] ^ SB[ny * pw + wi]) & kBit1) +
-             ((c ^ SA[nz * pw + wi] ^ SB[nz * pw + wi]) & kBit1);
-      if (++since == 40) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) diff[b] += (acc >> (8 * b + 1)) & 0x7Fu;
-        acc = 0;
-        since = 0;
+  const long long Nb = 3LL * N;
+  long long local = 0;
+  const int64_t first = ((int64_t)blockIdx.x * (kLinkThreads / 32) + warp) * kLinkPairsPerWarp;
+  for (int64_t j = first; j < min(first + kLinkPairsPerWarp, (int64_t)pairs); ++j) {
+    const uint32_t* ra = A.spins[cur] + j * g.sw;
+    const uint32_t* rb = B.spins[cur] + j * g.sw;
+    for (int k = lane; k < row_words; k += 32) c[k] = k < nw ? ra[k] ^ rb[k] : 0u;
+    __syncwarp();
+    // the first plane again from bit N on (word nw - 1 holds the last N mod 32 sites)
+    const int at = N >> 5, sh = N & 31, words = (L * L + sh + 31) / 32;
+    uint32_t ext[2] = {0u, 0u};  // L <= 16: at most nine words of the first plane
+    for (int q = 0; q < 2; ++q) {
+      const int k = lane + 32 * q;
+      if (k < words) {
+        const uint32_t lo = k > 0 ? c[k - 1] : 0u, hi = c[k];
+        ext[q] = sh ? __funnelshift_l(lo, hi, sh) : hi;
       }
     }
-    long long local = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      diff[b] += (acc >> (8 * b + 1)) & 0x7Fu;
-      if (4 * wi + b < pairs) {
-        const long long QL = Nb - 2LL * diff[b];
-        atomicAdd(&qh[((QL + Nb) * (long long)(g.q_bins - 1) + Nb) / (2 * Nb)], 1u);
-        local += QL;
-      }
+    __syncwarp();
+    for (int q = 0; q < 2; ++q) {
+      const int k = lane + 32 * q;
+      if (k < words) c[at + k] = k == 0 && sh ? (c[at] & ((1u << sh) - 1u)) | (ext[q] & ~((1u << sh) - 1u)) : ext[q];
     }
-    atomicAdd(reinterpret_cast<unsigned long long*>(&ssum), (unsigned long long)local);
+    __syncwarp();
+    int diff = 0;
+    for (int k = lane; k < nw; k += 32) {
+      const int n0 = 32 * k;
+      const uint32_t x = c[k];
+      const uint32_t valid = n0 + 32 <= N ? ~0u : (1u << (N - n0)) - 1u;
+      // edge sites' neighbours lie L - 1 (L (L - 1)) bits back; before bit 0 there are none
+      const int bx = n0 - (L - 1), by = n0 - L * (L - 1);
+      const uint32_t ex = bx >= 0 ? bits_at(c, bx) : c[0] << (unsigned)(-bx);
+      const uint32_t ey = by >= 0 ? bits_at(c, by) : by > -32 ? c[0] << (unsigned)(-by) : 0u;
+      const uint32_t sx = (bits_at(c, n0 + 1) & ~wx[k]) | (ex & wx[k]);
+      const uint32_t sy = (bits_at(c, n0 + L) & ~wy[k]) | (ey & wy[k]);
+      const uint32_t sz = bits_at(c, n0 + L * L);
+      diff += __popc((x ^ sx) & valid) + __popc((x ^ sy) & valid) + __popc((x ^ sz) & valid);
+    }
+    diff = warp_sum(diff);
+    if (lane == 0) {
+      const long long QL = Nb - 2LL * diff;
+      atomicAdd(&qh[((QL + Nb) * (long long)(g.q_bins - 1) + Nb) / (2 * Nb)], 1u);
+      local += QL;
+    }
+    __syncwarp();  // c is read before the next pair overwrites it
   }
+  if (lane == 0 && local) atomicAdd(reinterpret_cast<unsigned long long*>(&ssum), (unsigned long long)local);
   __syncthreads();
   unsigned long long* row = qlhist + (size_t)t * g.q_bins;
   for (int i = threadIdx.x; i < g.q_bins; i += blockDim.x)
@@ -653,12 +659,6 @@ __global__ void k_g_link(RunGeom g, GArgs a, int cur, int t, unsigned long long*
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-
-int launch_g_energy_init(const RunGeom& g, PopDev* pops, int cur, const int32_t* Jq, void* stream) {
-  dim3 grid(blocks_for(g.pitch / 4, 128), g.n_pop);
-  k_g_energy_init<<<grid, 128, 0, (cudaStream_t)stream>>>(g, gpack(pops, g.n_pop), cur, Jq);
-  return (int)cudaGetLastError();
-}
 
 int launch_g_resample(const RunGeom& g, PopDev* pops, int cur, int t, const double* wtab, int32_t* status,
                       void* stream) {
@@ -750,8 +750,10 @@ int launch_g_measure(const RunGeom& g, PopDev* pops, int cur, int t, unsigned lo
   k_g_finish<<<1, g.n_pop, 0, s>>>(g, a, t);
   k_g_count_E0<<<dim3(g.n_measure_blocks, g.n_pop), kMeasureThreads, 0, s>>>(g, a, t);
   if (g.n_pop == 2) {
-    const size_t smem = sizeof(unsigned int) * (size_t)g.q_bins;
-    k_g_link<<<blocks_for(g.pitch / 4, 256), 256, smem, s>>>(g, a, cur, t, qlhist);
+    const int warps = kLinkThreads / 32;
+    const size_t smem =
+        sizeof(uint32_t) * ((size_t)g.q_bins + 2 * ((size_t)g.N + 31) / 32 + 1 + (size_t)warps * link_row_words(g.N, g.L));
+    k_g_link<<<blocks_for(g.R_cap, warps * kLinkPairsPerWarp), kLinkThreads, smem, s>>>(g, a, cur, t, qlhist);
   }
   return (int)cudaGetLastError();
 }

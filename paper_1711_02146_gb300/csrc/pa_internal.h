@@ -51,7 +51,11 @@ struct GRec {
 
 // Device buffers of one population.
 struct PopDev {
-  int8_t* spins[2];     // [N][pitch] int8 +1/-1, site-major (replicas contiguous)
+  // One bit per spin, replica-major (pa_bits.cuh): slot j is the row of sw words at
+  // j sw, rows [0, pitch).  Each buffer is N pitch bytes; what follows the rows, and the
+  // whole of the buffer that does not hold the current population, is scratch (the
+  // site-major words of the large-lattice sweep, the int8 spins of a read-out).
+  uint32_t* spins[2];
   int32_t* labels[2];   // [R_cap] family labels
   int32_t* levels;      // [pitch] energy level k of each slot of the current population
   int32_t* counts;      // [R_cap] copy numbers of the old slots
@@ -80,10 +84,15 @@ struct PopDev {
   uint32_t key_init[2];
 };
 
+// Words per replica row of the spin arrays (pa_bits.cuh): whole words, and whole
+// 32-byte sectors beyond 64 sites.
+constexpr int spin_words(int N) { return N <= 64 ? (N + 31) / 32 : ((N + 255) / 256) * 8; }
+
 // Geometry of one run.
 struct RunGeom {
   int32_t L, N, n_levels;
-  int64_t pitch;        // bytes per site row of the spin arrays (multiple of 1024)
+  int64_t pitch;        // slots of the population arrays (R_cap rounded up to a multiple of 1024)
+  int32_t sw;           // words per replica row of the spin arrays (spin_words(N))
   int32_t R;            // target population
   int32_t R_cap;
   int32_t n_pop;
@@ -144,8 +153,18 @@ constexpr int kSlotsPerCountBlock = 1024;
 
 // ---- launchers (pa_kernels.cu / pa_sweep.cu); each returns a cudaError_t as int ----
 int launch_init_couplings(const RunGeom& g, uint64_t disorder_seed, int8_t* J, uint32_t* jtab, void* stream);
-int launch_init_population(const RunGeom& g, PopDev* pops, int cur, void* stream);
-int launch_levels_and_hist(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, void* stream);
+// The initial spins into spins[buf] and labels (slot numbers) into labels[1 - buf]: the
+// step-0 sweep launch (no sweeps, every slot its own parent) takes the spins from
+// there into the other buffer and counts the energy levels.
+int launch_init_population(const RunGeom& g, PopDev* pops, int buf, void* stream);
+// Read-outs of the current population: the spins of slots [first, first + n) of the rows
+// `spins` as int8 +1 / -1, replica-major [n][N] or site-major [N][ld] (ld a multiple of
+// 32, >= n), and the reverse of the latter, into slots [0, n).
+int launch_unpack_replicas(const RunGeom& g, const uint32_t* spins, int64_t first, int64_t n, int8_t* out,
+                           void* stream);
+int launch_unpack_rows(const RunGeom& g, const uint32_t* spins, int64_t first, int64_t n, int64_t ld, int8_t* out,
+                       void* stream);
+int launch_pack_rows(const RunGeom& g, const int8_t* in, int64_t n, int64_t ld, uint32_t* spins, void* stream);
 int launch_reweight(const RunGeom& g, PopDev* pops, const double* w, int t, void* stream);
 // Polls after which a look-back wait of the single-pass resampling gives up.
 constexpr int kLookbackSpins = 1 << 20;
@@ -161,6 +180,9 @@ int launch_resample(const RunGeom& g, PopDev* pops, int cur, int t, int32_t* sta
                     void* stream);
 int launch_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, int n_sweeps,
                  const uint32_t met_thr[3], void* stream);
+// Step 0: energy levels, histogram and families of the initial population in
+// spins[1], which moves to spins[0].
+int launch_sweep_initial(const RunGeom& g, PopDev* pops, const uint32_t* jtab, void* stream);
 // Family statistics of step t (sum of eta^2, families, sum of nu ln nu) into the step
 // records; the +-1 shared-memory sweep does the same in its epilogue.
 int launch_families(const RunGeom& g, PopDev* pops, int cur, int t, void* stream);
@@ -169,11 +191,13 @@ int launch_families(const RunGeom& g, PopDev* pops, int cur, int t, void* stream
 int launch_family_hist(const RunGeom& g, PopDev* pops, int pop, int cur, int t, void* stream);
 // Gaussian-coupling model (pa_gauss.cu, and k_sweep_g in pa_sweep.cu)
 int launch_scan_scatter(const RunGeom& g, PopDev* pops, int cur, int t, int32_t* status, void* stream);
-int launch_g_energy_init(const RunGeom& g, PopDev* pops, int cur, const int32_t* Jq, void* stream);
 int launch_g_resample(const RunGeom& g, PopDev* pops, int cur, int t, const double* wtab, int32_t* status,
                       void* stream);
 int launch_g_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
                    const uint32_t* gtab, int t, int n_sweeps, void* stream);
+// Step 0: the energies of the initial population in spins[1], which moves to spins[0].
+int launch_g_sweep_initial(const RunGeom& g, PopDev* pops, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
+                           void* stream);
 // The expected culling fraction of population 0 for the weight tables wtab, into
 // rec[t].eps_expected (also overwrites the step-t weights, sums and tables, which the
 // resampling recomputes): one evaluation of the adaptive bisection.
@@ -198,6 +222,7 @@ int launch_g_bisect_fused(const RunGeom& g, PopDev* pops, int t, double* tables,
                           unsigned long long* bar, double* b, double target, int halvings, int n_blocks,
                           int withheld, void* stream);
 int launch_overlap(const RunGeom& g, PopDev* pops, int cur, int t, unsigned long long* qhist, void* stream);
+int overlap_blocks(const RunGeom& g);  // blocks of the overlap of one pair of populations
 
 // ---- a batch advanced by one launch per kernel and temperature step (pa_batch) ----
 // Every population of every run of the batch is a unit; a round takes each unit's
@@ -276,8 +301,11 @@ bool lattice_supported(int L);      // every lattice a run accepts (even L <= kM
 // S half-sweep launches in place, energy levels.
 int launch_sweep_global(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, int n_sweeps,
                         const uint32_t met_thr[3], void* stream);
+// The same for step 0 (no sweeps): levels and histogram of the initial population in
+// spins[1], which moves to spins[0].
+int launch_sweep_global_initial(const RunGeom& g, PopDev* pops, const uint32_t* jtab, void* stream);
 // Sharded runs: the copies of population pop's resampling written out as replicas,
-// new[n][j] = old[n][parents[j]] for j < rec[t].R_tilde (pa_sweep_global.cu).
+// row j of the new buffer = row parents[j] of the old one for j < rec[t].R_tilde.
 int launch_copy_parents(const RunGeom& g, PopDev* pops, int pop, int cur, int t, void* stream);
 // Family runs of one rank's slots (labels[cur][0, rec[t].R_tilde)): the first and
 // the last run (they may continue on other ranks) into edge = {has slots, first

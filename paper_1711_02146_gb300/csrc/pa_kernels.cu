@@ -1,13 +1,10 @@
 // pa_kernels.cu — initialisation, reweighting, resampling, family and overlap
 // kernels of the population annealing step (Amey & Machta, §II, §III.A).
 //
-// Spin storage: int8 +1 (0x01) / -1 (0xFF), site-major: row n holds all slots of
-// site n contiguously (pitch bytes), so one 32-bit word carries four replicas
-// of one site.  For two spins a, b of that encoding a ^ b is 0x00 when equal and
-// 0xFE when different; XOR with a coupling mask (0xFE for J = -1, else 0) gives
-// 0xFE exactly for an unsatisfied bond, and bit 1 of each byte counts it.
+// Spins are one bit each, replica-major rows of sw words (pa_bits.cuh).
 #include <cuda_runtime.h>
 
+#include "pa_bits.cuh"
 #include "pa_device.cuh"
 #include "pa_family.cuh"
 #include "pa_internal.h"
@@ -24,7 +21,6 @@ static PopArgs pack(const PopDev* pops, int n_pop) {
   return a;
 }
 
-constexpr uint32_t kBit1 = 0x02020202u;
 constexpr int kScatterOwn = 16;  // copies a thread writes alone; larger families are written by the warp
 
 // ---------------------------------------------------------------- init (a0)
@@ -47,76 +43,100 @@ __global__ void k_init_couplings(int N, uint32_t k0, uint32_t k1, int8_t* J, uin
 
 // Initial spins: slot j at site n is +1 if bit 0 of word (j & 3) of Philox at
 // counter (n, 0, j >> 2, 0) is 0, else -1, j the global slot (slot_base + local
-// slot); slots past the initial population are padded with +1.
-__global__ void k_init_population(RunGeom g, PopArgs a, int cur) {
+// slot); slots past the initial population are padded with +1.  A thread draws one
+// word of 32 sites of four replicas (a block serves the four), lanes along a row.
+__global__ void k_init_population(RunGeom g, PopArgs a, int buf) {
   const int pop = blockIdx.y;
   const PopDev& P = a.p[pop];
-  const int64_t words = g.pitch / 4;
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= words * g.N) return;
-  const int n = (int)(gid / words);
-  const uint32_t wi = (uint32_t)(gid % words);
-  const uint32_t gw = (uint32_t)(g.slot_base / 4) + wi;  // global word (slot_base is a multiple of 4)
-  const uint4 r = philox4x32_10(make_uint4((uint32_t)n, 0u, gw, 0u), P.key_init[0], P.key_init[1]);
-  uint32_t out = 0;
+  const int64_t wi = gid / g.sw;  // slots 4 wi .. 4 wi + 3
+  if (wi >= g.pitch / 4) return;
+  const int blk = (int)(gid % g.sw);
+  const uint32_t gw = (uint32_t)(g.slot_base / 4) + (uint32_t)wi;  // slot_base is a multiple of 4
+  uint32_t out[4] = {0u, 0u, 0u, 0u};
+  const int n_sites = min(32, g.N - 32 * blk);  // <= 0 in the padding of a row
+  for (int i = 0; i < n_sites; ++i) {
+    const uint4 r = philox4x32_10(make_uint4((uint32_t)(32 * blk + i), 0u, gw, 0u), P.key_init[0], P.key_init[1]);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) out[b] |= (word_of(r, b) & 1u) << i;
+  }
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
-    const int64_t j = 4 * (int64_t)wi + b;
-    const uint32_t byte = (j < g.n_init && (word_of(r, b) & 1u)) ? 0xFFu : 0x01u;
-    out |= byte << (8 * b);
+    const int64_t j = 4 * wi + b;
+    P.spins[buf][j * g.sw + blk] = j < g.n_init ? out[b] : 0u;
+    if (blk == 0 && j < g.n_init) P.labels[1 - buf][j] = (int32_t)(g.slot_base + j);
   }
-  reinterpret_cast<uint32_t*>(P.spins[cur] + (size_t)n * g.pitch)[wi] = out;
-  if (n == 0) {
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int64_t j = 4 * (int64_t)wi + b;
-      if (j < g.n_init) P.labels[cur][j] = (int32_t)(g.slot_base + j);
-    }
-  }
-  if (n == 0 && wi == 0) P.rec[0].R_tilde = g.n_init;
+  if (gid == 0) P.rec[0].R_tilde = g.n_init;
 }
 
-// Energy level (unsatisfied bonds) of every slot from scratch, and the level
-// histogram of step t.  One thread per word (four replicas).
-__global__ void k_levels_and_hist(RunGeom g, PopArgs a, int cur, const uint32_t* __restrict__ jtab, int t) {
-  const int pop = blockIdx.y;
-  const PopDev& P = a.p[pop];
-  const int R = P.rec[t].R_tilde;
-  const int wi = blockIdx.x * blockDim.x + threadIdx.x;
-  if (4 * wi >= R) return;
-  const int L = g.L;
-  const uint32_t* S = reinterpret_cast<const uint32_t*>(P.spins[cur]);
-  const int64_t pw = g.pitch / 4;
-  int cnt[4] = {0, 0, 0, 0};
-  uint32_t acc = 0;
-  int since = 0;
-  for (int n = 0; n < g.N; ++n) {
-    const int x = n % L, y = (n / L) % L, z = n / (L * L);
-    const int nx = (x + 1 == L ? 0 : x + 1) + L * (y + L * z);
-    const int ny = x + L * ((y + 1 == L ? 0 : y + 1) + L * z);
-    const int nz = x + L * (y + L * (z + 1 == L ? 0 : z + 1));
-    const uint32_t s = S[n * pw + wi];
-    acc += ((s ^ S[nx * pw + wi] ^ jtab[4 * n + 0]) & kBit1) + ((s ^ S[ny * pw + wi] ^ jtab[4 * n + 1]) & kBit1) +
-           ((s ^ S[nz * pw + wi] ^ jtab[4 * n + 2]) & kBit1);
-    if (++since == 40) {
+// ---------------------------------------------------------------- read-outs
+
+// int8 spins, replica-major [n][N]: eight sites (one byte of a row; N is a multiple
+// of 8) per thread, reads and writes both along the rows.
+__global__ void __launch_bounds__(256) k_unpack_replicas(RunGeom g, const uint32_t* __restrict__ spins, int64_t first,
+                                                         int64_t n, int8_t* out) {
+  const int oct = g.N / 8;
+  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (o >= n * oct) return;
+  const int64_t j = o / oct;
+  const int k = (int)(o % oct);
+  const uint32_t x = reinterpret_cast<const uint8_t*>(spins + (first + j) * g.sw)[k];
+  reinterpret_cast<uint2*>(out)[o] = make_uint2(spins_to_bytes(x), spins_to_bytes(x >> 4));
+}
+
+// int8 spins, site-major rows of ld bytes: a thread transposes 32 sites of 32 slots.
+__global__ void __launch_bounds__(128) k_unpack_rows(RunGeom g, const uint32_t* __restrict__ spins, int64_t first,
+                                                     int64_t n, int64_t ld, int8_t* out) {
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // slots 32 w .. 32 w + 31
+  if (32 * w >= n) return;
+  const int blk = blockIdx.y;
+  uint32_t m[32];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) cnt[b] += (acc >> (8 * b)) & 0xFFu;
-      acc = 0;
-      since = 0;
+  for (int i = 0; i < 32; ++i) m[i] = 32 * w + i < n ? spins[(first + 32 * w + i) * g.sw + blk] : 0u;
+  transpose32(m);
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    const int site = 32 * blk + i;
+    if (site >= g.N) break;
+    uint4* o = reinterpret_cast<uint4*>(out + (size_t)site * ld + 32 * w);
+    o[0] = make_uint4(spins_to_bytes(m[i]), spins_to_bytes(m[i] >> 4), spins_to_bytes(m[i] >> 8),
+                      spins_to_bytes(m[i] >> 12));
+    o[1] = make_uint4(spins_to_bytes(m[i] >> 16), spins_to_bytes(m[i] >> 20), spins_to_bytes(m[i] >> 24),
+                      spins_to_bytes(m[i] >> 28));
+  }
+}
+
+// The reverse, into slots [0, n): whole rows, their padding included.
+__global__ void __launch_bounds__(128) k_pack_rows(RunGeom g, const int8_t* __restrict__ in, int64_t n, int64_t ld,
+                                                   uint32_t* spins) {
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (32 * w >= n) return;
+  const int blk = blockIdx.y;
+  uint32_t m[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    const int site = 32 * blk + i;
+    m[i] = 0u;
+    if (site < g.N) {
+      const uint4* v = reinterpret_cast<const uint4*>(in + (size_t)site * ld + 32 * w);
+      const uint4 lo = v[0], hi = v[1];
+      m[i] = bytes_to_spins(lo.x) | bytes_to_spins(lo.y) << 4 | bytes_to_spins(lo.z) << 8 |
+             bytes_to_spins(lo.w) << 12 | bytes_to_spins(hi.x) << 16 | bytes_to_spins(hi.y) << 20 |
+             bytes_to_spins(hi.z) << 24 | bytes_to_spins(hi.w) << 28;
     }
   }
+  transpose32(m);
 #pragma unroll
-  for (int b = 0; b < 4; ++b) cnt[b] += (acc >> (8 * b)) & 0xFFu;
-  uint32_t* hist = P.hist + (size_t)t * g.n_levels;
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int j = 4 * wi + b;
-    if (j < R) {
-      const int k = cnt[b] >> 1;
-      P.levels[j] = k;
-      atomicAdd(&hist[k], 1u);
-    }
-  }
+  for (int i = 0; i < 32; ++i)
+    if (32 * w + i < n) spins[(32 * w + i) * g.sw + blk] = m[i];
+}
+
+// Row j of the new buffer = row parents[j] of the old one (sharded runs).
+__global__ void __launch_bounds__(256) k_copy_parents(RunGeom g, PopDev P, int cur, int t) {
+  const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t j = o / g.sw;
+  if (j >= P.rec[t].R_tilde) return;
+  P.spins[1 - cur][o] = P.spins[cur][(int64_t)P.parents[j] * g.sw + o % g.sw];
 }
 
 // ---------------------------------------------------------------- reweight (a4)
@@ -601,45 +621,45 @@ __global__ void __launch_bounds__(1024) k_entropy_of_sizes(const int32_t* eta, c
 // ---------------------------------------------------------------- overlap (a8)
 
 // q between slot j of population 0 and slot j of population 1, j < min(R~0, R~1):
-// Q = N - 2 (sites that differ); bin = ((Q + N)(B - 1) + N) div 2N.
-// Block `blk` of the pairs of populations A, B (256 words of four slots each).
+// Q = N - 2 (sites that differ), the bits set in the XOR of the two rows; bin =
+// ((Q + N)(B - 1) + N) div 2N.  overlap_lanes lanes share a pair, 16 bytes each at a
+// time (8 and 4 for rows of two words and one), so that a warp reads whole sectors.  Bound by HBM: 2 rows per pair (with int8
+// site-major spins the same histogram read eight times the bytes, 143 us at L = 8 and
+// 1e5 pairs).  Block `blk` takes the pairs [blk p, (blk + 1) p), p = 256 / lanes.
+__host__ __device__ inline int overlap_lanes(int sw) { return sw >= 32 ? 8 : sw >= 16 ? 4 : sw >= 8 ? 2 : 1; }
+
 __device__ __forceinline__ void overlap_pops(const RunGeom& g, const PopDev& A, const PopDev& B, int cur, int t,
                                              unsigned long long* qhist, unsigned int* qh, int blk) {
   __shared__ unsigned int small_sh;
   const int pairs = min(A.rec[t].R_tilde, B.rec[t].R_tilde);
+  const int lanes = overlap_lanes(g.sw);
   for (int i = threadIdx.x; i < g.q_bins; i += blockDim.x) qh[i] = 0u;
   if (threadIdx.x == 0) small_sh = 0u;
   __syncthreads();
-  const int wi = blk * blockDim.x + threadIdx.x;
-  if (4 * wi < pairs) {
-    const uint32_t* SA = reinterpret_cast<const uint32_t*>(A.spins[cur]);
-    const uint32_t* SB = reinterpret_cast<const uint32_t*>(B.spins[cur]);
-    const int64_t pw = g.pitch / 4;
-    int diff[4] = {0, 0, 0, 0};
-    uint32_t acc = 0;
-    int since = 0;
-    for (int n = 0; n < g.N; ++n) {
-      acc += ((SA[n * pw + wi] ^ SB[n * pw + wi]) >> 1) & 0x01010101u;
-      if (++since == 255) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) diff[b] += (acc >> (8 * b)) & 0xFFu;
-        acc = 0;
-        since = 0;
+  const int part = (int)threadIdx.x % lanes;
+  const int64_t j = (int64_t)blk * (blockDim.x / lanes) + threadIdx.x / lanes;
+  int diff = 0;
+  if (j < pairs) {
+    const uint32_t* ra = A.spins[cur] + j * g.sw;
+    const uint32_t* rb = B.spins[cur] + j * g.sw;
+    if (g.sw % 4 == 0) {
+      const uint4* va = reinterpret_cast<const uint4*>(ra);
+      const uint4* vb = reinterpret_cast<const uint4*>(rb);
+      for (int k = part; k < g.sw / 4; k += lanes) {
+        const uint4 x = va[k], y = vb[k];
+        diff += __popc(x.x ^ y.x) + __popc(x.y ^ y.y) + __popc(x.z ^ y.z) + __popc(x.w ^ y.w);
       }
+    } else {
+      for (int k = part; k < g.sw; k += lanes) diff += __popc(ra[k] ^ rb[k]);
     }
-    unsigned int small = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      diff[b] += (acc >> (8 * b)) & 0xFFu;
-      if (4 * wi + b < pairs) {
-        const long long Q = (long long)g.N - 2LL * diff[b];
-        const long long bin = ((Q + g.N) * (long long)(g.q_bins - 1) + g.N) / (2LL * g.N);
-        atomicAdd(&qh[bin], 1u);
-        const long long aq = Q < 0 ? -Q : Q;
-        small += (5 * aq <= g.N) ? 1u : 0u;
-      }
-    }
-    if (small) atomicAdd(&small_sh, small);
+  }
+  for (int o = lanes / 2; o > 0; o >>= 1) diff += __shfl_xor_sync(0xffffffffu, diff, o);
+  if (j < pairs && part == 0) {
+    const long long Q = (long long)g.N - 2LL * diff;
+    const long long bin = ((Q + g.N) * (long long)(g.q_bins - 1) + g.N) / (2LL * g.N);
+    atomicAdd(&qh[bin], 1u);
+    const long long aq = Q < 0 ? -Q : Q;
+    if (5 * aq <= g.N) atomicAdd(&small_sh, 1u);
   }
   __syncthreads();
   unsigned long long* row = qhist + (size_t)t * g.q_bins;
@@ -681,16 +701,34 @@ int launch_init_couplings(const RunGeom& g, uint64_t disorder_seed, int8_t* J, u
   return (int)cudaGetLastError();
 }
 
-int launch_init_population(const RunGeom& g, PopDev* pops, int cur, void* stream) {
-  const int64_t total = (g.pitch / 4) * g.N;
+int launch_init_population(const RunGeom& g, PopDev* pops, int buf, void* stream) {
+  const int64_t total = (g.pitch / 4) * g.sw;
   dim3 grid(grid_for(total, 256), g.n_pop);
-  k_init_population<<<grid, 256, 0, (cudaStream_t)stream>>>(g, pack(pops, g.n_pop), cur);
+  k_init_population<<<grid, 256, 0, (cudaStream_t)stream>>>(g, pack(pops, g.n_pop), buf);
   return (int)cudaGetLastError();
 }
 
-int launch_levels_and_hist(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, void* stream) {
-  dim3 grid(grid_for(g.pitch / 4, 128), g.n_pop);
-  k_levels_and_hist<<<grid, 128, 0, (cudaStream_t)stream>>>(g, pack(pops, g.n_pop), cur, jtab, t);
+int launch_unpack_replicas(const RunGeom& g, const uint32_t* spins, int64_t first, int64_t n, int8_t* out,
+                           void* stream) {
+  k_unpack_replicas<<<grid_for(n * (g.N / 8), 256), 256, 0, (cudaStream_t)stream>>>(g, spins, first, n, out);
+  return (int)cudaGetLastError();
+}
+
+int launch_unpack_rows(const RunGeom& g, const uint32_t* spins, int64_t first, int64_t n, int64_t ld, int8_t* out,
+                       void* stream) {
+  const dim3 grid(grid_for((n + 31) / 32, 128), (g.N + 31) / 32);
+  k_unpack_rows<<<grid, 128, 0, (cudaStream_t)stream>>>(g, spins, first, n, ld, out);
+  return (int)cudaGetLastError();
+}
+
+int launch_pack_rows(const RunGeom& g, const int8_t* in, int64_t n, int64_t ld, uint32_t* spins, void* stream) {
+  const dim3 grid(grid_for((n + 31) / 32, 128), g.sw);
+  k_pack_rows<<<grid, 128, 0, (cudaStream_t)stream>>>(g, in, n, ld, spins);
+  return (int)cudaGetLastError();
+}
+
+int launch_copy_parents(const RunGeom& g, PopDev* pops, int pop, int cur, int t, void* stream) {
+  k_copy_parents<<<grid_for((int64_t)g.R_cap * g.sw, 256), 256, 0, (cudaStream_t)stream>>>(g, pops[pop], cur, t);
   return (int)cudaGetLastError();
 }
 
@@ -784,10 +822,12 @@ int launch_group_advance(int32_t* round, void* stream) {
   return (int)cudaGetLastError();
 }
 
+int overlap_blocks(const RunGeom& g) { return grid_for((int64_t)g.R_cap * overlap_lanes(g.sw), 256); }
+
 int launch_overlap(const RunGeom& g, PopDev* pops, int cur, int t, unsigned long long* qhist, void* stream) {
   if (g.n_pop != 2) return 0;
   const size_t smem = sizeof(unsigned int) * (size_t)g.q_bins;
-  k_overlap<<<grid_for(g.pitch / 4, 256), 256, smem, (cudaStream_t)stream>>>(g, pack(pops, 2), cur, t, qhist);
+  k_overlap<<<overlap_blocks(g), 256, smem, (cudaStream_t)stream>>>(g, pack(pops, 2), cur, t, qhist);
   return (int)cudaGetLastError();
 }
 

@@ -225,6 +225,33 @@ int copy_h2d(pa_ctx* c, void* dst, const void* src, size_t bytes) {
   return rc == PA_OK ? cuda_status(cudaStreamSynchronize(c->stream)) : rc;
 }
 
+// Spins of slots [first, first + n) of the rows `spins` to a host array of N rows of n
+// int8 spins (site-major: checkpoints and rank exchanges), and of such an array into
+// slots [0, n): expanded to and packed from bits on the device, in `scratch` (N rows
+// of n rounded up to 32 bytes: a spin buffer that holds nothing of use).
+int64_t row_bytes(int64_t n) { return (n + 31) / 32 * 32; }
+
+int copy_rows_d2h(pa_ctx* c, const uint32_t* spins, int64_t first, int64_t n, int8_t* scratch, void* host) {
+  const RunGeom& g = c->g;
+  const size_t ld = (size_t)row_bytes(n);
+  int rc = pa::launch_unpack_rows(g, spins, first, n, (int64_t)ld, scratch, c->stream) == 0 ? PA_OK : PA_ERR_CUDA;
+  c->stats.d2h_bytes += (int64_t)g.N * n;
+  if (rc == PA_OK)
+    rc = cuda_status(cudaMemcpy2DAsync(host, (size_t)n, scratch, ld, (size_t)n, (size_t)g.N, cudaMemcpyDeviceToHost,
+                                       c->stream));
+  return rc == PA_OK ? cuda_status(cudaStreamSynchronize(c->stream)) : rc;
+}
+
+int copy_rows_h2d(pa_ctx* c, uint32_t* spins, int64_t n, int8_t* scratch, const void* host) {
+  const RunGeom& g = c->g;
+  const size_t ld = (size_t)row_bytes(n);
+  c->stats.h2d_bytes += (int64_t)g.N * n;
+  int rc = cuda_status(cudaMemcpy2DAsync(scratch, ld, host, (size_t)n, (size_t)n, (size_t)g.N, cudaMemcpyHostToDevice,
+                                         c->stream));
+  if (rc == PA_OK) rc = pa::launch_pack_rows(g, scratch, n, (int64_t)ld, spins, c->stream) == 0 ? PA_OK : PA_ERR_CUDA;
+  return rc == PA_OK ? cuda_status(cudaStreamSynchronize(c->stream)) : rc;
+}
+
 // Stream-ordered host-to-device copy; the caller keeps src alive until the stream
 // has been synchronised.
 int copy_async(pa_ctx* c, void* dst, const void* src, size_t bytes) {
@@ -682,8 +709,9 @@ int measure(pa_ctx* c, int t) {
     PhaseTimer pt(c, PA_PHASE_FAMILY, 3);
     rc = launch_rc(pa::launch_g_measure(c->g, c->pops, c->cur, t, c->qlhist, c->stream));
   }
-  // the +-1 shared-memory sweep adds the family statistics of steps t >= 1 itself
-  const bool in_sweep = c->model == PA_MODEL_PM1 && t > 0 && pa::sweep_supported(c->g.L);
+  // the +-1 shared-memory sweep adds the family statistics itself (step 0: its launch
+  // without sweeps)
+  const bool in_sweep = c->model == PA_MODEL_PM1 && pa::sweep_supported(c->g.L);
   if (rc == PA_OK && !in_sweep) {
     PhaseTimer pt(c, PA_PHASE_FAMILY, 1);
     rc = launch_rc(pa::launch_families(c->g, c->pops, c->cur, t, c->stream));
@@ -791,6 +819,7 @@ void init_run(pa_ctx* c, const pa_config* cfg, int64_t R_cap) {
   g.N = cfg->L * cfg->L * cfg->L;
   g.n_levels = 3 * g.N + 1;
   g.pitch = ((R_cap + 1023) / 1024) * 1024;  // a whole number of sweep tiles (<= 1024 replicas)
+  g.sw = pa::spin_words(g.N);
   g.R = (int32_t)cfg->R;
   g.R_cap = (int32_t)R_cap;
   g.n_pop = cfg->n_pop;
@@ -826,7 +855,9 @@ int layout_buffers(pa_ctx* c) {
   for (int p = 0; p < g.n_pop && rc == PA_OK; ++p) {
     PopDev& P = c->pops[p];
     for (int b = 0; b < 2 && rc == PA_OK; ++b) {
-      rc = dalloc(c, &P.spins[b], (size_t)g.N * (size_t)g.pitch);
+      int8_t* buf = nullptr;  // a byte per spin: rows of bits, and scratch behind them (PopDev)
+      rc = dalloc(c, &buf, (size_t)g.N * (size_t)g.pitch);
+      P.spins[b] = reinterpret_cast<uint32_t*>(buf);
       rc = rc ? rc : dalloc(c, &P.labels[b], (size_t)g.pitch);
     }
     rc = rc ? rc : dalloc(c, &P.levels, (size_t)g.pitch);
@@ -1164,8 +1195,8 @@ int create_run_impl(const pa_config* cfg, void* cuda_stream, pa_ctx** out, bool 
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->J, 0, (size_t)3 * g.N, s));
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->jtab, 0, sizeof(uint32_t) * 4 * g.N, s));
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->qlhist, 0, sizeof(unsigned long long) * T * g.q_bins, s));
-    if (rc == PA_OK) rc = launch_rc(pa::launch_init_population(g, c->pops, 0, s));
-    if (rc == PA_OK) rc = launch_rc(pa::launch_g_energy_init(g, c->pops, 0, c->Jq, s));
+    if (rc == PA_OK) rc = launch_rc(pa::launch_init_population(g, c->pops, 1, s));
+    if (rc == PA_OK) rc = launch_rc(pa::launch_g_sweep_initial(g, c->pops, c->jtab, c->Jq, c->Jtot, s));
   } else {
     if (!c->adaptive) {
       const std::vector<double> d = distinct_dbetas(c->betas);
@@ -1179,8 +1210,10 @@ int create_run_impl(const pa_config* cfg, void* cuda_stream, pa_ctx** out, bool 
         rc = copy_async(c, c->wtables[bits_of(d[0])], c->wtables_host.data(), sizeof(double) * c->wtables_host.size());
     }
     if (rc == PA_OK) rc = launch_rc(pa::launch_init_couplings(g, cfg->disorder_seed, c->J, c->jtab, s));
-    if (rc == PA_OK) rc = launch_rc(pa::launch_init_population(g, c->pops, 0, s));
-    if (rc == PA_OK) rc = launch_rc(pa::launch_levels_and_hist(g, c->pops, 0, c->jtab, 0, s));
+    if (rc == PA_OK) rc = launch_rc(pa::launch_init_population(g, c->pops, 1, s));
+    if (rc == PA_OK)
+      rc = launch_rc(pa::sweep_supported(g.L) ? pa::launch_sweep_initial(g, c->pops, c->jtab, s)
+                                              : pa::launch_sweep_global_initial(g, c->pops, c->jtab, s));
   }
   if (rc == PA_OK) rc = measure(c, 0);
   if (rc == PA_OK) record_step_done(c, 0);
@@ -1259,7 +1292,7 @@ int pa_step(pa_ctx* c) try {
       PhaseTimer pt(c, PA_PHASE_SWEEP, c->g.n_pop * (c->g.tail_shape >= 0 ? 2 : 1));
       rc = launch_rc(pa::launch_sweep(c->g, c->pops, c->cur, c->jtab, t, c->sweeps[(size_t)t], met, s));
     } else if (rc == PA_OK) {  // lattices beyond a shared-memory tile: sweeps in global memory
-      PhaseTimer pt(c, PA_PHASE_SWEEP, c->g.n_pop * (1 + 2 * c->sweeps[(size_t)t]) + 1);
+      PhaseTimer pt(c, PA_PHASE_SWEEP, c->g.n_pop * (5 + 2 * c->sweeps[(size_t)t]));
       rc = launch_rc(pa::launch_sweep_global(c->g, c->pops, c->cur, c->jtab, t, c->sweeps[(size_t)t], met, s));
     }
   }
@@ -1476,14 +1509,11 @@ int pa_get_replicas(pa_ctx* c, int32_t pop, int64_t first, int64_t n, int8_t* sp
   const RunGeom& g = c->g;
   const PopDev& P = c->pops[pop];
   if (spins) {
-    std::vector<int8_t> tmp((size_t)g.N * (size_t)n);
-    c->stats.d2h_bytes += (int64_t)g.N * n;
-    rc = cuda_status(cudaMemcpy2DAsync(tmp.data(), (size_t)n, P.spins[c->cur] + first, (size_t)g.pitch, (size_t)n,
-                                       (size_t)g.N, cudaMemcpyDeviceToHost, c->stream));
-    if (rc == PA_OK) rc = cuda_status(cudaStreamSynchronize(c->stream));
+    // expanded on the device into the buffer that does not hold the population
+    int8_t* out = reinterpret_cast<int8_t*>(P.spins[1 - c->cur]);
+    rc = launch_rc(pa::launch_unpack_replicas(g, P.spins[c->cur], first, n, out, c->stream));
+    if (rc == PA_OK) rc = copy_d2h(c, spins, out, (size_t)g.N * (size_t)n);
     if (rc != PA_OK) return fail(c, rc);
-    for (int64_t j = 0; j < n; ++j)
-      for (int s = 0; s < g.N; ++s) spins[(size_t)j * g.N + s] = tmp[(size_t)s * n + j];
   }
   if (labels) {
     rc = copy_d2h(c, labels, P.labels[c->cur] + first, sizeof(int32_t) * n);
@@ -1720,10 +1750,7 @@ int pa_checkpoint(pa_ctx* c, void* buf, size_t cap, size_t* size) try {
     else
       get(P.hist, sizeof(uint32_t) * (size_t)(t + 1) * (size_t)g.n_levels);
     if (rc == PA_OK && R) {
-      c->stats.d2h_bytes += (int64_t)(g.N * R);
-      rc = cuda_status(cudaMemcpy2DAsync(o, R, P.spins[c->cur], (size_t)g.pitch, R, (size_t)g.N,
-                                         cudaMemcpyDeviceToHost, c->stream));
-      if (rc == PA_OK) rc = cuda_status(cudaStreamSynchronize(c->stream));
+      rc = copy_rows_d2h(c, P.spins[c->cur], 0, (int64_t)R, reinterpret_cast<int8_t*>(P.spins[1 - c->cur]), o);
     }
     o += (size_t)g.N * R;
     get(P.labels[c->cur], sizeof(int32_t) * R);
@@ -1808,12 +1835,8 @@ int pa_restore(const pa_config* cfg, const void* buf, size_t size, void* cuda_st
       put(P.grec, sizeof(pa::GRec) * (size_t)(t + 1));
     else
       put(P.hist, sizeof(uint32_t) * (size_t)(t + 1) * (size_t)g.n_levels);
-    if (rc == PA_OK) {
-      c->stats.h2d_bytes += (int64_t)(g.N * R);
-      rc = cuda_status(cudaMemcpy2DAsync(P.spins[0], (size_t)g.pitch, in, R, R, (size_t)g.N,
-                                         cudaMemcpyHostToDevice, c->stream));
-      if (rc == PA_OK) rc = cuda_status(cudaStreamSynchronize(c->stream));
-    }
+    if (rc == PA_OK)
+      rc = copy_rows_h2d(c, P.spins[0], (int64_t)R, reinterpret_cast<int8_t*>(P.spins[1]), in);
     in += (size_t)g.N * R;
     put(P.labels[0], sizeof(int32_t) * R);
     if (gauss)
@@ -2167,9 +2190,8 @@ int shard_exchange(pa_shard* s, int p, const std::vector<int64_t>& off, const st
     sp.assign((size_t)(N * std::max<int64_t>(n, 1)), 0);
     lb.assign((size_t)std::max<int64_t>(n, 1), 0);
     if (n == 0) return PA_OK;
-    int rc = cuda_status(cudaMemcpy2DAsync(sp.data(), (size_t)n, P.spins[1 - c->cur] + a, (size_t)g.pitch, (size_t)n,
-                                           (size_t)N, cudaMemcpyDeviceToHost, c->stream));
-    if (rc == PA_OK) rc = cuda_status(cudaStreamSynchronize(c->stream));
+    // the copies are in the other buffer; the old population is no longer needed
+    int rc = copy_rows_d2h(c, P.spins[1 - c->cur], a, n, reinterpret_cast<int8_t*>(P.spins[c->cur]), sp.data());
     if (rc == PA_OK) rc = copy_d2h(c, lb.data(), P.labels[1 - c->cur] + a, sizeof(int32_t) * (size_t)n);
     return rc;
   };
@@ -2223,8 +2245,7 @@ int shard_exchange(pa_shard* s, int p, const std::vector<int64_t>& off, const st
   }
   if (rc != PA_OK) return rc;
   if (n_new > 0) {
-    rc = cuda_status(cudaMemcpy2DAsync(P.spins[c->cur], (size_t)g.pitch, rs.data(), (size_t)n_new, (size_t)n_new,
-                                       (size_t)N, cudaMemcpyHostToDevice, c->stream));
+    rc = copy_rows_h2d(c, P.spins[c->cur], n_new, reinterpret_cast<int8_t*>(P.spins[1 - c->cur]), rs.data());
     if (rc == PA_OK) rc = copy_h2d(c, P.labels[1 - c->cur], rl.data(), sizeof(int32_t) * (size_t)n_new);
     std::vector<int32_t> iota((size_t)n_new);
     for (int64_t j = 0; j < n_new; ++j) iota[(size_t)j] = (int32_t)j;
@@ -2556,7 +2577,7 @@ int group_build(Group* G) {
     }
     if (c->g.n_pop == 2) {
       pairs[q] = GroupPair{first_unit[(size_t)i], first_unit[(size_t)i] + 1, c->qhist};
-      pair_off[q + 1] = pair_off[q] + (int32_t)((c->g.pitch / 4 + 255) / 256);
+      pair_off[q + 1] = pair_off[q] + (int32_t)overlap_blocks(c->g);
       ++q;
     }
   }

@@ -8,10 +8,13 @@
 //      c = (x + y + z) & 1, colour 0 then colour 1; the neighbours of a site all
 //      have the other colour, so all sites of one colour update independently),
 //   3. counts each replica's energy and adds the tile to the histogram of step t,
-//   4. writes the tile to the new population buffer (int8 +1 / -1),
+//   4. writes the tile to the new population buffer,
 //   5. (+-1 couplings) adds the families of its slots to the step's family
 //      statistics (§III.A), so the step needs no family launch of its own.
-// HBM traffic is one read and one write of the tile per step, whatever S is.
+// HBM traffic is one read and one write of the tile per step, whatever S is, at one
+// bit per spin (pa_bits.cuh): a replica is a row of spin_words(N) words, and the
+// gather and the store each transpose 32 x 32 bits in registers between 32 rows and
+// 32 site words.
 //
 // +-1 couplings (k_sweep): bit-sliced tiles.  Word w of a site row holds slots
 // tile0 + 32w + b as bit b (set for spin -1), so one 32-bit logic instruction
@@ -42,45 +45,27 @@
 
 #include <algorithm>
 
+#include "pa_bits.cuh"
 #include "pa_device.cuh"
 #include "pa_family.cuh"
 #include "pa_internal.h"
+#include "pa_metropolis.cuh"
 
 namespace pa {
 
-constexpr uint32_t kM0 = 0xD2511F53u;
-constexpr uint32_t kM1 = 0xCD9E8D57u;
-
-struct SweepArgs {
+struct SweepArgs : MetropolisArgs {
   PopDev pop;
   const uint32_t* jtab;  // [N][4] forward-bond masks (non-zero for J = -1)
-  int64_t pitch;
   int32_t n_levels;
   int32_t t;
   int32_t cur;
   int32_t n_sweeps;
   int32_t slot_base;  // global slot of local slot 0 (Philox groups are global); 0 for a whole population
   int32_t fam;        // 1: add the tile's families to the step record (not for one rank's share)
+  int32_t fresh;      // 1: step 0, every slot is its own parent
   // this launch's first local slot (tile 0 of the grid), and the split of a two-launch
   // sweep: slots below `split` in tiles of tj_main, the rest in tiles of tj_tail
   int32_t tile_base, split, tj_main, tj_tail;
-  uint32_t thr4, thr8, thr12;
-  uint32_t k0[10];  // Metropolis round keys of this population
-  uint32_t k1[10];
-  // +-1: plane p's threshold bit as a function of the unsatisfied-bond count u
-  // (bits u0, u1; u = 0, 1, 2): T(u) = bit 31 - p of thr(u) as an all-zero / all-one
-  // word, stored as tm[p] = {T(0), T(0) ^ T(1), T(0) ^ T(2)}, so that the bit of a
-  // replica is tm[p][0] ^ (u0 & tm[p][1]) ^ (u1 & tm[p][2]) (u >= 3 never compares)
-  uint32_t tm[32][4];
-  uint32_t live[4];    // +-1: the same form of "thr(u) > 0" (a replica with thr(u) = 0 never flips)
-};
-
-// Per-site shared-memory record: the six bond masks of the site (all ones for
-// J = -1), and the site/step-dependent parts of Philox rounds 2-3 for h = n >> 1
-// (the third, lo(M0 h), is one multiply and is recomputed).
-struct __align__(16) SiteRec {
-  uint32_t jxp, jxm, jyp, jym;
-  uint32_t jzp, jzm, ua, ub;
 };
 
 // Nibble tiles of the Gaussian kernel: 8 replicas per word.
@@ -98,36 +83,6 @@ struct SweepShape {
   static_assert(L % 2 == 0 && L / 2 <= 8, "even L up to 16");
   static_assert(NP % 2 == 0 && (ROWS / 2) % (NP / 2) == 0, "row partitions must split each parity class");
 };
-
-// 32 x 32 -> 64-bit product as one wide multiply (2.4 % faster sweep than the
-// separate high and low products).
-__device__ __forceinline__ void mulhilo(uint32_t m, uint32_t a, uint32_t& hi, uint32_t& lo) {
-  uint64_t p;
-  asm("mul.wide.u32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(m));
-  hi = (uint32_t)(p >> 32);
-  lo = (uint32_t)p;
-}
-
-// Per-thread, per-half-sweep part of rounds 1-3 of one group g.
-struct ThreadPhilox {
-  uint32_t ta;   // lo(M1 g): XORed with the site's ua to give round-2 word 0
-  uint32_t tb;   // hi(M0 A1) ^ k1_2: XORed with lo(M0 h) to give round-2 word 2
-  uint32_t tdk;  // lo(M0 A1) ^ k1_3: round-3 word 2 is hi(M0 A2) ^ tdk
-};
-
-__device__ __forceinline__ ThreadPhilox thread_philox(uint32_t g, uint32_t q, const uint32_t* k0,
-                                                      const uint32_t* k1) {
-  uint32_t h1, l1;
-  mulhilo(kM1, g, h1, l1);
-  const uint32_t a1 = h1 ^ q ^ k0[0];
-  uint32_t ha, la;
-  mulhilo(kM0, a1, ha, la);
-  ThreadPhilox tp;
-  tp.ta = l1;
-  tp.tb = ha ^ k1[1];
-  tp.tdk = la ^ k1[2];
-  return tp;
-}
 
 // Row k of a partition: rows of one parity class (y + z) & 1 = p, interleaved
 // across the partitions of that class.
@@ -163,15 +118,18 @@ __device__ __forceinline__ void fill_row_table(int* rowtab, int tid, int nthread
   }
 }
 
-// int8 spins (0x01 / 0xFF) of four replicas -> nibbles 0..3 (bit 1 of a byte is the sign)
-__device__ __forceinline__ uint32_t bytes_to_nibbles(uint32_t w) {
-  const uint32_t b = (w >> 1) & 0x01010101u;
-  return (b & 1u) | ((b >> 4) & 0x10u) | ((b >> 8) & 0x100u) | ((b >> 12) & 0x1000u);
+// Bits 0..7 of x -> bit 0 of nibbles 0..7, and back.
+__device__ __forceinline__ uint32_t bits_to_nibbles(uint32_t x) {
+  x &= 0xffu;
+  x = (x | (x << 12)) & 0x000F000Fu;
+  x = (x | (x << 6)) & 0x03030303u;
+  return (x | (x << 3)) & 0x11111111u;
 }
-// nibbles 0..3 of x -> four int8 spins
-__device__ __forceinline__ uint32_t nibbles_to_bytes(uint32_t x) {
-  const uint32_t b = (x & 1u) | ((x & 0x10u) << 4) | ((x & 0x100u) << 8) | ((x & 0x1000u) << 12);
-  return b * 0xFEu + 0x01010101u;
+__device__ __forceinline__ uint32_t nibbles_to_bits(uint32_t x) {
+  x &= 0x11111111u;
+  x = (x | (x >> 3)) & 0x03030303u;
+  x = (x | (x >> 6)) & 0x000F000Fu;
+  return (x | (x >> 12)) & 0xffu;
 }
 
 // ---- phases of a tile: init_tables and publish_levels serve both kernels,
@@ -182,71 +140,38 @@ __device__ __forceinline__ uint32_t nibbles_to_bytes(uint32_t x) {
 template <int L>
 __device__ __forceinline__ void init_tables(const SweepArgs& a, SiteRec* recs, int tid, int nthreads) {
   constexpr int N = L * L * L;
-  const uint32_t* k0 = a.k0;
-  const uint32_t* k1 = a.k1;
   for (int n = tid; n < N; n += nthreads) {
-    const int x = n % L, y = (n / L) % L, z = n / (L * L);
-    const int nxm = (x == 0 ? L - 1 : x - 1) + L * (y + L * z);
-    const int nym = x + L * ((y == 0 ? L - 1 : y - 1) + L * z);
-    const int nzm = x + L * (y + L * (z == 0 ? L - 1 : z - 1));
-    SiteRec r;
-    r.jxp = a.jtab[4 * n + 0] ? ~0u : 0u;
-    r.jyp = a.jtab[4 * n + 1] ? ~0u : 0u;
-    r.jzp = a.jtab[4 * n + 2] ? ~0u : 0u;
-    r.jxm = a.jtab[4 * nxm + 0] ? ~0u : 0u;
-    r.jym = a.jtab[4 * nym + 1] ? ~0u : 0u;
-    r.jzm = a.jtab[4 * nzm + 2] ? ~0u : 0u;
-    const uint32_t h = (uint32_t)n >> 1;
-    uint32_t hi0, lo0, hi1, lo1;
-    mulhilo(kM0, h, hi0, lo0);
-    const uint32_t c1 = hi0 ^ (uint32_t)a.t ^ k1[0];
-    mulhilo(kM1, c1, hi1, lo1);
-    r.ua = hi1 ^ k0[1];
-    r.ub = lo1 ^ k0[2];
-    recs[n] = r;
+    recs[n] = site_record(L, n, a.jtab, (uint32_t)a.t, a);
   }
 }
 
-// Gather the tile's spins from the parents of its slots (nibble-packed).
-template <int L, int W, int NP>
-__device__ __forceinline__ void gather_tile(const SweepArgs& a, uint32_t* sp, int tile0, int R_new, int word,
-                                            int part) {
-  constexpr int N = L * L * L;
-  const PopDev& P = a.pop;
-  int par[8];
+// The parent (old slot) of new slot j, -1 past R~.
+__device__ __forceinline__ int parent_of(const SweepArgs& a, int j, int R_new) {
+  return j < R_new ? (a.fresh ? j : a.pop.parents[j]) : -1;
+}
+
+// Gather the tile's spins from the parents of its slots (nibble-packed): 32 slots
+// and 32 sites per thread, as gather_bits.
+template <int L, int W, int NT>
+__device__ __forceinline__ void gather_tile(const SweepArgs& a, uint32_t* sp, int tile0, int R_new) {
+  constexpr int N = Row<L>::N, SW = Row<L>::SW, NB = Row<L>::NB, GW = W / 4;  // groups of 32 slots
+  const uint32_t* src = a.pop.spins[a.cur];
+  for (int u = threadIdx.x; u < GW * NB; u += NT) {
+    const int gw = u % GW, blk = u / GW;
+    uint32_t m[32];
 #pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    const int j = tile0 + 8 * word + b;
-    par[b] = j < R_new ? P.parents[j] : -1;
-  }
-  bool contiguous = par[0] >= 0 && (par[0] & 7) == 0;
-#pragma unroll
-  for (int b = 1; b < 8; ++b) contiguous = contiguous && par[b] == par[0] + b;
-  const int8_t* src = P.spins[a.cur];
-  // rows are gathered GB at a time with every load issued before the first use
-  constexpr int GB = (N / NP) % 10 == 0 ? 10 : ((N / NP) % 8 == 0 ? 8 : ((N / NP) % 4 == 0 ? 4 : 1));
-  for (int n0 = part; n0 < N; n0 += NP * GB) {
-    uint2 vv[GB];
-#pragma unroll
-    for (int i = 0; i < GB; ++i) {
-      const int n = n0 + i * NP;
-      const int8_t* row = src + (size_t)(n < N ? n : 0) * a.pitch;
-      if (contiguous) {
-        vv[i] = *reinterpret_cast<const uint2*>(row + par[0]);
-      } else {
-        uint32_t lo = 0, hi = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          lo |= (par[b] >= 0 ? (uint32_t)(uint8_t)row[par[b]] : 0x01u) << (8 * b);
-          hi |= (par[b + 4] >= 0 ? (uint32_t)(uint8_t)row[par[b + 4]] : 0x01u) << (8 * b);
-        }
-        vv[i] = make_uint2(lo, hi);
-      }
+    for (int i = 0; i < 32; ++i) {
+      const int p = parent_of(a, tile0 + 32 * gw + i, R_new);
+      m[i] = p >= 0 ? src[(size_t)p * SW + blk] : 0u;
     }
+    transpose32(m);
 #pragma unroll
-    for (int i = 0; i < GB; ++i) {
-      const int n = n0 + i * NP;
-      if (n < N) sp[n * W + word] = bytes_to_nibbles(vv[i].x) | (bytes_to_nibbles(vv[i].y) << 16);
+    for (int i = 0; i < 32; ++i) {
+      const int n = 32 * blk + i;
+      if (N % 32 == 0 || n < N)
+        *reinterpret_cast<uint4*>(sp + n * W + 4 * gw) =
+            make_uint4(bits_to_nibbles(m[i]), bits_to_nibbles(m[i] >> 8), bits_to_nibbles(m[i] >> 16),
+                       bits_to_nibbles(m[i] >> 24));
     }
   }
 }
@@ -267,15 +192,24 @@ __device__ __forceinline__ void publish_levels(const SweepArgs& a, const int* ec
   }
 }
 
-// Write the tile back as int8 +1 (0x01) / -1 (0xFF).
-template <int L, int W, int NP>
-__device__ __forceinline__ void store_tile(const SweepArgs& a, const uint32_t* sp, int tile0, int word, int part) {
-  constexpr int N = L * L * L;
-  int8_t* dst = a.pop.spins[1 - a.cur];
-  for (int n = part; n < N; n += NP) {
-    const uint32_t w = sp[n * W + word];
-    *reinterpret_cast<uint2*>(dst + (size_t)n * a.pitch + tile0 + 8 * word) =
-        make_uint2(nibbles_to_bytes(w), nibbles_to_bytes(w >> 16));
+// Write the tile back to the rows of its slots, their padding included.
+template <int L, int W, int NT>
+__device__ __forceinline__ void store_tile(const SweepArgs& a, const uint32_t* sp, int tile0) {
+  constexpr int N = Row<L>::N, SW = Row<L>::SW, GW = W / 4;
+  uint32_t* dst = a.pop.spins[1 - a.cur];
+  for (int u = threadIdx.x; u < GW * SW; u += NT) {
+    const int gw = u % GW, blk = u / GW;
+    uint32_t m[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      const int n = 32 * blk + i;
+      const uint4 v = n < N ? *reinterpret_cast<const uint4*>(sp + n * W + 4 * gw)
+                                           : make_uint4(0u, 0u, 0u, 0u);
+      m[i] = nibbles_to_bits(v.x) | nibbles_to_bits(v.y) << 8 | nibbles_to_bits(v.z) << 16 | nibbles_to_bits(v.w) << 24;
+    }
+    transpose32(m);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) dst[(size_t)(tile0 + 32 * gw + i) * SW + blk] = m[i];
   }
 }
 
@@ -317,60 +251,6 @@ struct BitShape {
   static_assert(NP % 2 == 0 && (ROWS / 2) % (NP / 2) == 0, "row partitions must split each parity class");
   static_assert(1024 % TJ == 0, "a tile never crosses the 1024-slot pitch unit");
 };
-
-__device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a ^ b)); }
-
-// One Philox block (rounds 3..10 from the hoisted parts) of site h, uc = lo(M0 h),
-// for the thread's group of block index b (its ThreadPhilox tp).
-__device__ __forceinline__ void philox_block(uint32_t uc, const SiteRec& sr, const ThreadPhilox& tp, const uint32_t* k0,
-                                             const uint32_t* k1, uint32_t (&w)[4]) {
-  uint32_t hh, l, h2, l2;
-  mulhilo(kM1, tp.tb ^ uc, hh, l);
-  mulhilo(kM0, sr.ua ^ tp.ta, h2, l2);
-  w[0] = hh ^ sr.ub;
-  w[1] = l;
-  w[2] = h2 ^ tp.tdk;
-  w[3] = l2;
-#pragma unroll
-  for (int rr = 3; rr < 10; ++rr) {  // rounds 4..10 (key index rr)
-    mulhilo(kM1, w[2], hh, l);
-    mulhilo(kM0, w[0], h2, l2);
-    const uint32_t n0 = hh ^ w[1] ^ k0[rr];
-    const uint32_t n2 = h2 ^ w[3] ^ k1[rr];
-    w[0] = n0;
-    w[1] = l;
-    w[2] = n2;
-    w[3] = l2;
-  }
-}
-
-// The plane's threshold bit of each replica of a word (SweepArgs::tm), from bits
-// u0, u1 of its unsatisfied-bond count.
-__device__ __forceinline__ uint32_t threshold_bits(const uint32_t* tm, uint32_t u0, uint32_t u1) {
-  return tm[0] ^ (u0 & tm[1]) ^ (u1 & tm[2]);
-}
-
-// One plane of the comparison uniform < threshold for the 32 replicas of a word,
-// most significant plane first: r holds the plane's bit of every replica's
-// uniform.  eq: replicas whose uniform has matched its threshold so far; acc:
-// replicas decided below it.
-__device__ __forceinline__ void compare_plane(uint32_t r, uint32_t u0, uint32_t u1, const uint32_t* tm, uint32_t& eq,
-                                              uint32_t& acc) {
-  const uint32_t t = threshold_bits(tm, u0, u1);
-  acc |= eq & t & ~r;
-  eq &= ~(r ^ t);
-}
-
-// One plane of the same comparison taken least significant plane first, as the
-// borrow of a bit-sliced subtraction r - thr: after the planes p..7, lt holds the
-// replicas whose bits p..7 of r are below those of thr, same those whose bits
-// p..7 are equal.
-__device__ __forceinline__ void borrow_plane(uint32_t r, uint32_t u0, uint32_t u1, const uint32_t* tm, uint32_t& lt,
-                                             uint32_t& same) {
-  const uint32_t t = threshold_bits(tm, u0, u1);
-  lt = (~r & t) | (~(r ^ t) & lt);
-  same &= ~(r ^ t);
-}
 
 // One half-sweep of the rows of partition `part` (parity class p, colour sites at
 // x = X0 mod 2).  spw points at this thread's word of site 0; tp[b] are the
@@ -455,20 +335,8 @@ template <int W>
 __device__ __forceinline__ void finish_deferred(uint32_t* sp, const SiteRec* recs, const Deferred d, uint32_t q,
                                                 uint32_t gbase, const SweepArgs& a) {
   const int n = (int)(d.loc & 0xffffu), word = (int)(d.loc >> 16);
-  const uint32_t u0 = d.u0, u1 = d.u1;
-  uint32_t eq = d.eq, acc = 0;
-  const uint32_t g8 = 8u * (gbase + (uint32_t)word);
-  const uint32_t uc = kM0 * ((uint32_t)n >> 1);
-  const SiteRec sr = recs[n];
-#pragma unroll 1
-  for (int b = 2; b < 8 && eq; ++b) {
-    const ThreadPhilox tb = thread_philox(g8 + (uint32_t)b, q, a.k0, a.k1);
-    uint32_t w[4];
-    philox_block(uc, sr, tb, a.k0, a.k1, w);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) compare_plane(w[i], u0, u1, a.tm[4 * b + i], eq, acc);
-  }
-  sp[n * W + word] ^= acc;
+  sp[n * W + word] ^=
+      compare_rest(d.eq, d.u0, d.u1, (uint32_t)n, recs[n], 8u * (gbase + (uint32_t)word), q, a);
 }
 
 // One half-sweep of the rows of partition `part`, as sweep_rows_bits, for shapes
@@ -507,36 +375,17 @@ __device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const
       const int xp = x == L - 1 ? 0 : x + 1, xm = x == 0 ? L - 1 : x - 1;
       const SiteRec sr = rr[x];
       const uint32_t s0 = p0[x * W];
-      const uint32_t b0 = s0 ^ p0[xp * W] ^ sr.jxp, b1 = s0 ^ p0[xm * W] ^ sr.jxm;
-      const uint32_t b2 = s0 ^ pyp[x * W] ^ sr.jyp, b3 = s0 ^ pym[x * W] ^ sr.jym;
-      const uint32_t b4 = s0 ^ pzp[x * W] ^ sr.jzp, b5 = s0 ^ pzm[x * W] ^ sr.jzm;
-      const uint32_t sa = b0 ^ b1 ^ b2, ca = majority(b0, b1, b2);
-      const uint32_t sb = b3 ^ b4 ^ b5, cb = majority(b3, b4, b5);
-      const uint32_t u0 = sa ^ sb, k2 = sa & sb;
-      const uint32_t u1 = ca ^ cb ^ k2, u2 = majority(ca, cb, k2);
-      const uint32_t always = u2 | (u1 & u0);  // u >= 3: dE <= 0
-      // replicas to compare: u = 0, 1, 2 (dE = 12, 8, 4) with thr(u) > 0
-      const uint32_t cmp = ~always & threshold_bits(a.live, u0, u1);
-      uint32_t lt = 0, eq = cmp;
-      const uint32_t uc = kM0 * (h0 + (uint32_t)xh);  // lo(M0 h), h = n >> 1
-      {
-        uint32_t w0[4], w1[4];
-        philox_block(uc, sr, tp[0], a.k0, a.k1, w0);
-        philox_block(uc, sr, tp[1], a.k0, a.k1, w1);
-        // bits 31..24 of each uniform against those of its threshold, lowest plane first
-#pragma unroll
-        for (int i = 3; i >= 0; --i) borrow_plane(w1[i], u0, u1, a.tm[4 + i], lt, eq);
-#pragma unroll
-        for (int i = 3; i >= 0; --i) borrow_plane(w0[i], u0, u1, a.tm[i], lt, eq);
-      }
-      p0[x * W] = s0 ^ ((cmp & lt) | always);
+      const BondCount c = bond_count(s0, sr, p0[xp * W], p0[xm * W], pyp[x * W], pym[x * W], pzp[x * W], pzm[x * W], a);
+      uint32_t lt, eq;
+      compare_planes8(kM0 * (h0 + (uint32_t)xh), sr, tp, c, a, lt, eq);  // lo(M0 h), h = n >> 1
+      p0[x * W] = s0 ^ (lt | c.always);
       const unsigned dm = __ballot_sync(0xffffffffu, eq != 0u);
       if (eq) {
         Deferred d;
         d.loc = (uint32_t)(rL + x) | ((uint32_t)word << 16);
         d.eq = eq;
-        d.u0 = u0;
-        d.u1 = u1;
+        d.u0 = c.u0;
+        d.u1 = c.u1;
         dq[(head + cnt + __popc(dm & below)) & (kQueueCap - 1)] = d;
       }
       cnt += __popc(dm);
@@ -556,32 +405,48 @@ __device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const
 
 // Gather the tile's spins from the parents of its slots into bit words; spar
 // holds the tile's parents (-1 past R~), slot i at index 33 (i >> 5) + (i & 31).
-template <int L, int W, int NP>
-__device__ __forceinline__ void gather_bits(const SweepArgs& a, uint32_t* sp, const int* spar, int word, int part) {
-  constexpr int N = L * L * L;
-  int par[32];
+// A thread takes 32 slots (one word of the tile) and BW words of their rows, 32 BW
+// sites: BW loads of each row, a transpose, 32 BW words of the tile.  Consecutive
+// threads take consecutive words of a site row, so the shared-memory stores have no
+// bank conflicts; the rows are read in pieces of 4 BW bytes, a sector's other pieces
+// by other warps at the same time (L1).  BW = 2 where 64 words fit the registers.
+template <int L, int W, int NT, int MB>
+struct RowMove : Row<L> {
+  using Row<L>::SW;
+  using Row<L>::NB;
+  static constexpr int BW = SW % 2 == 0 && NT * MB <= 640 ? 2 : 1;
+  static constexpr int GATHER_UNITS = W * ((NB + BW - 1) / BW);
+  static constexpr int STORE_UNITS = W * (SW / BW);  // the padding of a row too: its bits stay 0
+};
+
+template <int L, int W, int NT, int MB>
+__device__ __forceinline__ void gather_bits(const SweepArgs& a, uint32_t* sp, const int* spar) {
+  using M = RowMove<L, W, NT, MB>;
+  const uint32_t* src = a.pop.spins[a.cur];
+  for (int u = threadIdx.x; u < M::GATHER_UNITS; u += NT) {
+    const int word = u % W, blk = u / W * M::BW;
+    uint32_t m[M::BW][32];
 #pragma unroll
-  for (int b = 0; b < 32; ++b) par[b] = spar[33 * word + b];
-  bool contiguous = par[0] >= 0 && (par[0] & 15) == 0;
-#pragma unroll
-  for (int b = 1; b < 32; ++b) contiguous = contiguous && par[b] == par[0] + b;
-  const int8_t* src = a.pop.spins[a.cur];
-  for (int n = part; n < N; n += NP) {
-    const int8_t* row = src + (size_t)n * a.pitch;
-    uint32_t bits = 0;
-    if (contiguous) {
-      const uint4* v = reinterpret_cast<const uint4*>(row + par[0]);
-      const uint4 lo = v[0], hi = v[1];
-      const uint32_t q8[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)  // bit 1 of each byte is the sign; gather four of them
-        bits |= ((((q8[i] >> 1) & 0x01010101u) * 0x01020408u) >> 24) << (4 * i);
-    } else {
-#pragma unroll
-      for (int b = 0; b < 32; ++b)
-        if (par[b] >= 0) bits |= (((uint32_t)(uint8_t)row[par[b]] >> 1) & 1u) << b;
+    for (int i = 0; i < 32; ++i) {
+      const int p = spar[33 * word + i];
+      const uint32_t* row = src + (size_t)(p >= 0 ? p : 0) * M::SW + blk;
+      if constexpr (M::BW == 2) {
+        const uint2 v = p >= 0 ? *reinterpret_cast<const uint2*>(row) : make_uint2(0u, 0u);
+        m[0][i] = v.x;
+        m[1][i] = v.y;
+      } else {
+        m[0][i] = p >= 0 ? *row : 0u;
+      }
     }
-    sp[n * W + word] = bits;
+#pragma unroll
+    for (int h = 0; h < M::BW; ++h) {
+      transpose32(m[h]);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int n = 32 * (blk + h) + i;
+        if (M::N % (32 * M::BW) == 0 || n < M::N) sp[n * W + word] = m[h][i];
+      }
+    }
   }
 }
 
@@ -631,22 +496,31 @@ __device__ __forceinline__ void count_levels_bits(const uint32_t* sp, const Site
   }
 }
 
-// Write the tile back as int8 +1 (0x01) / -1 (0xFF), 32 slots per word.
-template <int L, int W, int NP>
-__device__ __forceinline__ void store_bits(const SweepArgs& a, const uint32_t* sp, int tile0, int word, int part) {
-  constexpr int N = L * L * L;
-  int8_t* dst = a.pop.spins[1 - a.cur];
-  for (int n = part; n < N; n += NP) {
-    const uint32_t w = sp[n * W + word];
-    uint32_t q8[8];
+// Write the tile back to the rows of its slots, the gather's split reversed.
+template <int L, int W, int NT, int MB>
+__device__ __forceinline__ void store_bits(const SweepArgs& a, const uint32_t* sp, int tile0) {
+  using M = RowMove<L, W, NT, MB>;
+  uint32_t* dst = a.pop.spins[1 - a.cur];
+  for (int u = threadIdx.x; u < M::STORE_UNITS; u += NT) {
+    const int word = u % W, blk = u / W * M::BW;
+    uint32_t m[M::BW][32];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {  // four bits -> bit 0 of four bytes -> 0x01 / 0xFF
-      const uint32_t m = (((w >> (4 * i)) & 15u) * 0x00204081u) & 0x01010101u;
-      q8[i] = m * 0xFEu + 0x01010101u;
+    for (int h = 0; h < M::BW; ++h) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int n = 32 * (blk + h) + i;
+        m[h][i] = n < M::N ? sp[n * W + word] : 0u;
+      }
+      transpose32(m[h]);
     }
-    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)n * a.pitch + tile0 + 32 * word);
-    out[0] = make_uint4(q8[0], q8[1], q8[2], q8[3]);
-    out[1] = make_uint4(q8[4], q8[5], q8[6], q8[7]);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      uint32_t* row = dst + (size_t)(tile0 + 32 * word + i) * M::SW + blk;
+      if constexpr (M::BW == 2)
+        *reinterpret_cast<uint2*>(row) = make_uint2(m[0][i], m[1][i]);
+      else
+        *row = m[0][i];
+    }
   }
 }
 
@@ -730,9 +604,9 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int
   Deferred* dq = queues + (S::DEFER ? (tid >> 5) * kQueueCap : 0);
   init_tables<L>(a, recs, tid, NT);
   if constexpr (S::DEFER) fill_row_table<L, W, NP>(rowtab, tid, NT);
-  for (int i = tid; i < TJ; i += NT) slots[33 * (i >> 5) + (i & 31)] = tile0 + i < R_new ? a.pop.parents[tile0 + i] : -1;
+  for (int i = tid; i < TJ; i += NT) slots[33 * (i >> 5) + (i & 31)] = parent_of(a, tile0 + i, R_new);
   __syncthreads();
-  gather_bits<L, W, NP>(a, sp, slots, word, part);
+  gather_bits<L, W, NT, MB>(a, sp, slots);
   __syncthreads();
   for (int i = tid; i < S::SLOTS; i += NT) slots[i] = 0;
   __syncthreads();
@@ -767,7 +641,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int
   count_levels_bits<L, W, NP, S::CB>(sp, recs, slots, word, part);
   __syncthreads();
   publish_levels<TJ>(a, slots, tile0, R_new, tid, NT);
-  store_bits<L, W, NP>(a, sp, tile0, word, part);
+  store_bits<L, W, NT, MB>(a, sp, tile0);
   if (!a.fam) return;
   __syncthreads();  // every shared array is dead now: the family pass takes the space
   tile_families<TJ, NT>(a, reinterpret_cast<int*>(sm), tile0, R_new, tid);
@@ -785,47 +659,23 @@ __global__ void __launch_bounds__(NT, MB) k_sweep(const __grid_constant__ SweepA
 
 // The sweep arguments of population P at step t from buffer cur with thresholds
 // thr (dE = 4, 8, 12), as launch_sweep sets them for a run of one launch.
-__host__ __device__ inline void fill_sweep_args(SweepArgs& a, const PopDev& P, const uint32_t* jtab, int64_t pitch,
+__host__ __device__ inline void fill_sweep_args(SweepArgs& a, const PopDev& P, const uint32_t* jtab,
                                                 int n_levels, int t, int cur, int n_sweeps, int tj,
                                                 const uint32_t thr[3]) {
   a.pop = P;
-  uint32_t k0 = P.key_met[0], k1 = P.key_met[1];
-  for (int r = 0; r < 10; ++r) {
-    a.k0[r] = k0;
-    a.k1[r] = k1;
-    k0 += 0x9E3779B9u;
-    k1 += 0xBB67AE85u;
-  }
+  fill_metropolis(a, P.key_met, thr);
   a.jtab = jtab;
-  a.pitch = pitch;
   a.n_levels = n_levels;
   a.t = t;
   a.cur = cur;
   a.n_sweeps = n_sweeps;
   a.slot_base = 0;
   a.fam = 1;
+  a.fresh = 0;
   a.tile_base = 0;
   a.split = 0x7fffffff;
   a.tj_main = tj;
   a.tj_tail = tj;
-  a.thr4 = thr[0];
-  a.thr8 = thr[1];
-  a.thr12 = thr[2];
-  const uint32_t thr_u[3] = {thr[2], thr[1], thr[0]};  // u = 0, 1, 2: dE = 12, 8, 4
-  for (int p = 0; p < 32; ++p) {
-    uint32_t T[3];
-    for (int u = 0; u < 3; ++u) T[u] = ((thr_u[u] >> (31 - p)) & 1u) ? ~0u : 0u;
-    a.tm[p][0] = T[0];
-    a.tm[p][1] = T[0] ^ T[1];
-    a.tm[p][2] = T[0] ^ T[2];
-    a.tm[p][3] = 0u;
-  }
-  uint32_t live[3];
-  for (int u = 0; u < 3; ++u) live[u] = thr_u[u] ? ~0u : 0u;
-  a.live[0] = live[0];
-  a.live[1] = live[0] ^ live[1];
-  a.live[2] = live[0] ^ live[2];
-  a.live[3] = 0u;
 }
 
 // The sweeps of a batch's units of one lattice size and launch shape: unit list[k]
@@ -855,7 +705,7 @@ __global__ void __launch_bounds__(NT, MB)
     hdr[2] = R_new;
     if (tile0 < R_new) {
       const GroupStep& st = u.steps[t];
-      fill_sweep_args(sa, u.P, u.jtab, u.g.pitch, u.g.n_levels, t, u.cur0 ^ (r & 1), st.n_sweeps, TJ, st.thr);
+      fill_sweep_args(sa, u.P, u.jtab, u.g.n_levels, t, u.cur0 ^ (r & 1), st.n_sweeps, TJ, st.thr);
     }
   }
   __syncthreads();
@@ -1010,7 +860,7 @@ __global__ void __launch_bounds__(NT, MB) k_sweep_g(const __grid_constant__ GSwe
   init_tables<L>(a, recs, tid, NT);
   fill_row_table<L, W, NP>(rowtab, tid, NT);
   for (int i = tid; i < TJ; i += NT) ecnt[i] = 0;
-  gather_tile<L, W, NP>(a, sp, tile0, R_new, word, part);
+  gather_tile<L, W, NT>(a, sp, tile0, R_new);
   __syncthreads();
   const uint32_t slot0 = (uint32_t)tile0 + 8u * (uint32_t)word;  // the word's first replica
   const uint32_t g = slot0 >> 3;                                     // Philox group of its eight replicas
@@ -1034,7 +884,7 @@ __global__ void __launch_bounds__(NT, MB) k_sweep_g(const __grid_constant__ GSwe
     const int j = tile0 + i;
     if (j < R_new) a.pop.E64[j] = -ga.Jtot + 2 * ecnt[i];
   }
-  store_tile<L, W, NP>(a, sp, tile0, word, part);
+  store_tile<L, W, NT>(a, sp, tile0);
 }
 
 template <int L, int W, int NT, int MB>
@@ -1121,17 +971,18 @@ bool sweep_shape_info(int L, int i, SweepShapeInfo* out) {
   return true;
 }
 
-int launch_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, int n_sweeps,
-                 const uint32_t met_thr[3], void* stream) {
+static int sweep_launches(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, int n_sweeps,
+                          const uint32_t met_thr[3], bool fresh, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   const ShapeEntry* shape = shape_of(g.L, g.sweep_shape);
   if (!shape) return (int)cudaErrorInvalidValue;
   const ShapeEntry* tail = g.tail_shape >= 0 ? shape_of(g.L, g.tail_shape) : nullptr;
   for (int i = 0; i < g.n_pop; ++i) {
     SweepArgs args;
-    fill_sweep_args(args, pops[i], jtab, g.pitch, g.n_levels, t, cur, n_sweeps, 32 * shape->W, met_thr);
+    fill_sweep_args(args, pops[i], jtab, g.n_levels, t, cur, n_sweeps, 32 * shape->W, met_thr);
     args.slot_base = g.slot_base;
     args.fam = g.shard ? 0 : 1;
+    args.fresh = fresh ? 1 : 0;
     args.split = tail ? g.tail_from : 0x7fffffff;
     args.tj_tail = tail ? 32 * tail->W : 32 * shape->W;
     int e = shape->launch(g, args, s);
@@ -1142,6 +993,16 @@ int launch_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, 
     if (e != 0) return e;
   }
   return 0;
+}
+
+int launch_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, int t, int n_sweeps,
+                 const uint32_t met_thr[3], void* stream) {
+  return sweep_launches(g, pops, cur, jtab, t, n_sweeps, met_thr, false, stream);
+}
+
+int launch_sweep_initial(const RunGeom& g, PopDev* pops, const uint32_t* jtab, void* stream) {
+  const uint32_t none[3] = {0u, 0u, 0u};
+  return sweep_launches(g, pops, 1, jtab, 0, 0, none, true, stream);
 }
 
 int sweep_tile_slots(int L, int shape) {
@@ -1174,32 +1035,26 @@ void sweep_tail_plan(int L, int shape, int64_t R, int n_sm, int32_t* tail_shape,
   *tail_from = (int32_t)(full * slots * tj);
 }
 
-int launch_g_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
-                   const uint32_t* gtab, int t, int n_sweeps, void* stream) {
+static int g_sweep_launches(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq,
+                            long long Jtot, const uint32_t* gtab, int t, int n_sweeps, bool fresh, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   for (int i = 0; i < g.n_pop; ++i) {
     GSweepArgs ga;
     SweepArgs& args = ga.base;
     args.pop = pops[i];
-    uint32_t k0 = pops[i].key_met[0], k1 = pops[i].key_met[1];
-    for (int r = 0; r < 10; ++r) {
-      args.k0[r] = k0;
-      args.k1[r] = k1;
-      k0 += 0x9E3779B9u;
-      k1 += 0xBB67AE85u;
-    }
+    const uint32_t none[3] = {0u, 0u, 0u};  // its thresholds are in gtab
+    fill_metropolis(args, pops[i].key_met, none);
     args.jtab = jtab;
-    args.pitch = g.pitch;
     args.n_levels = g.n_levels;
     args.t = t;
     args.cur = cur;
     args.n_sweeps = n_sweeps;
     args.slot_base = 0;
     args.fam = 0;
+    args.fresh = fresh ? 1 : 0;
     args.tile_base = 0;
     args.split = 0x7fffffff;
     args.tj_main = args.tj_tail = 1;
-    args.thr4 = args.thr8 = args.thr12 = 0u;
     ga.gtab = gtab;
     ga.Jq = Jq;
     ga.Jtot = Jtot;
@@ -1218,6 +1073,16 @@ int launch_g_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab
     if (e != 0) return e;
   }
   return 0;
+}
+
+int launch_g_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
+                   const uint32_t* gtab, int t, int n_sweeps, void* stream) {
+  return g_sweep_launches(g, pops, cur, jtab, Jq, Jtot, gtab, t, n_sweeps, false, stream);
+}
+
+int launch_g_sweep_initial(const RunGeom& g, PopDev* pops, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
+                           void* stream) {
+  return g_sweep_launches(g, pops, 1, jtab, Jq, Jtot, nullptr, 0, 0, true, stream);
 }
 
 }  // namespace pa
