@@ -19,7 +19,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpa.so")
 OBJDIR = os.path.join(HERE, "_build")
-SOURCES = ["pa_kernels.cu", "pa_sweep.cu", "pa_sweep_global.cu", "pa_gauss.cu", "pa_microbench.cu", "pa_noalloc.cu",
+SOURCES = ["pa_sweep_l10.cu", "pa_sweep_l6.cu", "pa_sweep_l2.cu", "pa_sweep_l8.cu", "pa_sweep_l12.cu", "pa_sweep_l14.cu",
+           "pa_sweep_gauss.cu", "pa_sweep.cu", "pa_kernels.cu", "pa_sweep_global.cu", "pa_gauss.cu", "pa_microbench.cu", "pa_noalloc.cu",
            "pa_runtime.cpp", "pa_serve.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

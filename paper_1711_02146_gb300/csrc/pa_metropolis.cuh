@@ -21,6 +21,10 @@ struct MetropolisArgs {
   // replica is tm[p][0] ^ (u0 & tm[p][1]) ^ (u1 & tm[p][2]) (u >= 3 never compares)
   uint32_t tm[32][4];
   uint32_t live[4];    // +-1: the same form of "thr(u) > 0" (a replica with thr(u) = 0 never flips)
+  // Leading zero bits of the thresholds, for the comparison's cheaper forms: `lead`
+  // Philox blocks (four planes each) in which every threshold's bits are 0, and the
+  // form of planes 0..7 (compare_planes8).
+  int32_t lead, form;
 };
 
 // Sets them from the population's key and the thresholds of dE = 4, 8, 12.
@@ -47,6 +51,11 @@ __host__ __device__ inline void fill_metropolis(MetropolisArgs& a, const uint32_
   a.live[1] = live[0] ^ live[1];
   a.live[2] = live[0] ^ live[2];
   a.live[3] = 0u;
+  int clz[2] = {0, 0};  // of thr(2) (dE = 4), the largest, and thr(1) (dE = 8)
+  for (int i = 0; i < 2; ++i)
+    while (clz[i] < 32 && !(thr[i] >> (31 - clz[i]) & 1u)) ++clz[i];
+  a.lead = clz[0] / 4;
+  a.form = clz[0] >= 8 ? 3 : clz[0] >= 4 && clz[1] >= 8 ? 2 : clz[0] >= 2 && clz[1] >= 4 ? 1 : 0;
 }
 
 // Per-site shared-memory record: the six bond masks of the site (all ones for
@@ -153,17 +162,6 @@ __device__ __forceinline__ void compare_plane(uint32_t r, uint32_t u0, uint32_t 
   eq &= ~(r ^ t);
 }
 
-// One plane of the same comparison taken least significant plane first, as the
-// borrow of a bit-sliced subtraction r - thr: after the planes p..7, lt holds the
-// replicas whose bits p..7 of r are below those of thr, same those whose bits
-// p..7 are equal.
-__device__ __forceinline__ void borrow_plane(uint32_t r, uint32_t u0, uint32_t u1, const uint32_t* tm, uint32_t& lt,
-                                             uint32_t& same) {
-  const uint32_t t = threshold_bits(tm, u0, u1);
-  lt = (~r & t) | (~(r ^ t) & lt);
-  same &= ~(r ^ t);
-}
-
 // Unsatisfied bonds of a site of 32 replicas: u's bits 0 and 1, the replicas that
 // always flip (u >= 3: dE <= 0), and those to compare (u = 0, 1, 2 with thr(u) > 0).
 struct BondCount {
@@ -190,19 +188,42 @@ __device__ __forceinline__ BondCount bond_count(uint32_t s0, const SiteRec& sr, 
 
 // Bit planes 0..7 (Philox blocks 0 and 1) of the comparison for the replicas in
 // c.cmp: lt = below the threshold in those planes, eq = equal so far.
+//
+// FORM says how many leading bits of the thresholds are 0 (thr(u) = 2^32 e^-beta(12-4u)
+// loses 5.8 beta, 11.5 beta and 17.3 beta leading bits at u = 2, 1, 0):
+//   3: all eight planes of every threshold are 0 (beta >= 1.39): a replica stays equal
+//      while its bits are 0 and is never below: one operation per two planes;
+//   2: planes 0..3 are 0, planes 4..7 only where u = 2 may not be (beta >= 0.69);
+//   1: planes 0, 1 are 0, 2, 3 only where u = 2 may not be (beta >= 0.35);
+//   0: any thresholds.
+// A plane costs four operations in general (threshold bit 2, borrow, equality), three
+// where only u = 2 has a threshold bit, half to one where none has: 34, 24, 15 and 4
+// per word for the forms 0 to 3, of some 150 per word and site in all.  With form 0 for
+// every step: L = 8, 201 temperatures to beta = 5, two populations of 1e5 97.9 ms, with
+// the forms 89.2; 64 runs of L = 4 to 10 on 101 temperatures 382 and 344 ms; L = 10,
+// R = 1e6 adaptive (most of its steps below beta = 0.7) 224.7 and 221.8 ms.
+template <int FORM>
 __device__ __forceinline__ void compare_planes8(uint32_t uc, const SiteRec& sr, const ThreadPhilox (&tp)[2],
                                                 const BondCount& c, const MetropolisArgs& a, uint32_t& lt,
                                                 uint32_t& eq) {
-  uint32_t w0[4], w1[4];
-  philox_block(uc, sr, tp[0], a.k0, a.k1, w0);
-  philox_block(uc, sr, tp[1], a.k0, a.k1, w1);
+  constexpr int ZERO = FORM == 3 ? 8 : FORM == 2 ? 4 : FORM == 1 ? 2 : 0;  // planes without any threshold bit
+  constexpr int TWO = FORM == 2 ? 8 : FORM == 1 ? 4 : ZERO;                // planes before this: only u = 2 has one
+  uint32_t w[2][4];
+  philox_block(uc, sr, tp[0], a.k0, a.k1, w[0]);
+  philox_block(uc, sr, tp[1], a.k0, a.k1, w[1]);
+  uint32_t same = c.cmp;
+#pragma unroll
+  for (int p = 0; p < ZERO; ++p) same &= ~w[p / 4][p & 3];
   lt = 0;
-  eq = c.cmp;
+  eq = same;
 #pragma unroll
-  for (int i = 3; i >= 0; --i) borrow_plane(w1[i], c.u0, c.u1, a.tm[4 + i], lt, eq);
-#pragma unroll
-  for (int i = 3; i >= 0; --i) borrow_plane(w0[i], c.u0, c.u1, a.tm[i], lt, eq);
-  lt &= c.cmp;
+  for (int p = 7; p >= ZERO; --p) {
+    const uint32_t r = w[p / 4][p & 3];
+    const uint32_t t = p < TWO ? c.u1 & a.tm[p][2] : threshold_bits(a.tm[p], c.u0, c.u1);
+    lt = (~r & t) | (~(r ^ t) & lt);
+    eq &= ~(r ^ t);
+  }
+  lt &= same;
 }
 
 // Bit planes 8.. (Philox blocks 2..7) of site n, record sr, for the replicas in eq of
@@ -216,6 +237,10 @@ __device__ __forceinline__ uint32_t compare_rest(uint32_t eq, uint32_t u0, uint3
     const ThreadPhilox tb = thread_philox(g8 + (uint32_t)b, q, a.k0, a.k1);
     uint32_t w[4];
     philox_block(uc, sr, tb, a.k0, a.k1, w);
+    if (b < a.lead) {  // no threshold bits in these planes
+      eq &= ~(w[0] | w[1] | w[2] | w[3]);
+      continue;
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) compare_plane(w[i], u0, u1, a.tm[4 * b + i], eq, acc);
   }

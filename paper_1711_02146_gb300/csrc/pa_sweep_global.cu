@@ -113,6 +113,7 @@ struct __align__(16) LatticeDeferred {
   uint32_t loc, eq, u0, u1;  // loc: lane of the owner | colour site in its row << 5
 };
 
+template <int FORM>
 __global__ void __launch_bounds__(kThreads) k_lattice_sweep(const __grid_constant__ LatticeArgs a, int q) {
   __shared__ LatticeDeferred queues[kWarps][64];
   const RunGeom& g = a.g;
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kThreads) k_lattice_sweep(const __grid_constan
       const uint32_t s0 = p0[at];
       b = bond_count(s0, sr, p0[xp * wp], p0[xm * wp], pyp[at], pym[at], pzp[at], pzm[at], a);
       uint32_t lt;
-      compare_planes8(kM0 * ((uint32_t)(r * L + x) >> 1), sr, tp, b, a, lt, eq);
+      compare_planes8<FORM>(kM0 * ((uint32_t)(r * L + x) >> 1), sr, tp, b, a, lt, eq);
       p0[at] = s0 ^ (lt | b.always);
     }
     const unsigned dm = __ballot_sync(0xffffffffu, eq != 0u);
@@ -250,8 +251,12 @@ int lattice_step(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, 
     k_lattice_records<<<(g.N + kThreads - 1) / kThreads, kThreads, 0, st>>>(a);
     k_lattice_transpose<false><<<tiles, kThreads, 0, st>>>(a);
     const int64_t threads = (int64_t)g.L * g.L * n_words;
-    for (int q = 0; q < 2 * n_sweeps; ++q)
-      k_lattice_sweep<<<(unsigned)((threads + kThreads - 1) / kThreads), kThreads, 0, st>>>(a, q);
+    const unsigned blocks = (unsigned)((threads + kThreads - 1) / kThreads);
+    auto* sweep = a.form == 3   ? k_lattice_sweep<3>
+                  : a.form == 2 ? k_lattice_sweep<2>
+                  : a.form == 1 ? k_lattice_sweep<1>
+                                : k_lattice_sweep<0>;
+    for (int q = 0; q < 2 * n_sweeps; ++q) sweep<<<blocks, kThreads, 0, st>>>(a, q);
     int e = (int)cudaMemsetAsync(pops[p].levels, 0, sizeof(int32_t) * (size_t)g.R_cap, st);
     if (e) return e;
     k_lattice_levels<<<dim3((n_words + kThreads - 1) / kThreads, (g.L * g.L + kLevelRows - 1) / kLevelRows), kThreads,

@@ -1,0 +1,701 @@
+// pa_sweep_tile.cuh — the +-1 Metropolis sweep kernels (the dominant cost of a PA step),
+// compiled per lattice size by the pa_sweep_l*.cu files.
+//
+// One CTA owns a tile of consecutive slots of the NEW population and all N sites
+// of those replicas in shared memory.  It
+//   1. gathers each slot's spins from its parent in the old population (the
+//      replica copy of the resampling, §II, fused into the load),
+//   2. runs S checkerboard Metropolis sweeps at beta_t in shared memory (colour
+//      c = (x + y + z) & 1, colour 0 then colour 1; the neighbours of a site all
+//      have the other colour, so all sites of one colour update independently),
+//   3. counts each replica's energy and adds the tile to the histogram of step t,
+//   4. writes the tile to the new population buffer,
+//   5. (+-1 couplings) adds the families of its slots to the step's family
+//      statistics (§III.A), so the step needs no family launch of its own.
+// HBM traffic is one read and one write of the tile per step, whatever S is, at one
+// bit per spin (pa_bits.cuh): a replica is a row of spin_words(N) words, and the
+// gather and the store each transpose 32 x 32 bits in registers between 32 rows and
+// 32 site words.
+//
+// +-1 couplings (k_sweep): bit-sliced tiles.  Word w of a site row holds slots
+// tile0 + 32w + b as bit b (set for spin -1), so one 32-bit logic instruction
+// tests a bond, adds a bit or takes a comparison step for 32 replicas.  Flipping
+// s_n costs dE = 12 - 4u, u = unsatisfied bonds at n; u comes from the six
+// bond bits by a tree of full adders as three bit planes.  u >= 3 (dE <= 0)
+// always flips; otherwise the flip is taken when the replica's 32-bit uniform r
+// is below thr(u) = floor(2^32 exp(-beta dE)).  r is the replica's bit column:
+// bit 31 - p of r is bit b of word p mod 4 of Philox4x32-10 at counter
+// (n >> 1, 2s + c, 8 (slot >> 5) + p / 4, t) keyed by (run_seed, Metropolis,
+// population), so one block gives four bit planes of 32 replicas' uniforms.
+// A replica is decided at the first plane, from the top, where its bit differs
+// from its threshold's (accepted if the threshold has the 1): two planes on
+// average.  Blocks 0 and 1 (planes 0..7) are always drawn and compared as one
+// 8-bit bit-sliced subtraction (its borrow is "below", plus an "equal so far"
+// mask); the words with replicas still equal draw further blocks on demand.
+//
+// Philox hoisting (same function, fewer multiplies): with counter words
+// (h, q, g, t) = (site, half-sweep, group, step), the round-1 and round-2
+// products depend either on the site and step only (tabulated once per launch
+// in shared memory) or on the thread and half-sweep only (registers), so each
+// block costs the 16 wide multiplies of rounds 3..10.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "pa_bits.cuh"
+#include "pa_device.cuh"
+#include "pa_family.cuh"
+#include "pa_internal.h"
+#include "pa_metropolis.cuh"
+
+namespace pa {
+
+struct SweepArgs : MetropolisArgs {
+  PopDev pop;
+  const uint32_t* jtab;  // [N][4] forward-bond masks (non-zero for J = -1)
+  int32_t n_levels;
+  int32_t t;
+  int32_t cur;
+  int32_t n_sweeps;
+  int32_t slot_base;  // global slot of local slot 0 (Philox groups are global); 0 for a whole population
+  int32_t fam;        // 1: add the tile's families to the step record (not for one rank's share)
+  int32_t fresh;      // 1: step 0, every slot is its own parent
+  // this launch's first local slot (tile 0 of the grid), and the split of a two-launch
+  // sweep: slots below `split` in tiles of tj_main, the rest in tiles of tj_tail
+  int32_t tile_base, split, tj_main, tj_tail;
+};
+
+// Row k of a partition: rows of one parity class (y + z) & 1 = p, interleaved
+// across the partitions of that class.
+template <int L, int NP>
+__device__ __forceinline__ int row_index(int part, int k, int p) {
+  constexpr int H = L / 2, PC = NP / 2;
+  const int i = (part % PC) + k * PC;  // index within the class
+  const int z = i / H;
+  const int y = 2 * (i % H) + ((p + z) & 1);
+  return y + L * z;
+}
+
+// Per partition and row (rows of the partition's parity class, row_index), the
+// word offsets of the row and of its four neighbour rows in a tile of W words per
+// site and the row's first site: {row, y+1, y-1, z+1, first site, z-1}.  A
+// thread's rows never change, so each tile fills this once.
+template <int L, int W, int NP>
+__device__ __forceinline__ void fill_row_table(int* rowtab, int tid, int nthreads) {
+  constexpr int RPP = L * L / NP;
+  for (int e = tid; e < NP * RPP; e += nthreads) {
+    const int pt = e / RPP, kr = e % RPP;
+    const int r = row_index<L, NP>(pt, kr, pt / (NP / 2));
+    const int y = r % L, z = r / L;
+    const int yp = y == L - 1 ? 0 : y + 1, ym = y == 0 ? L - 1 : y - 1;
+    const int zp = z == L - 1 ? 0 : z + 1, zm = z == 0 ? L - 1 : z - 1;
+    int* o = rowtab + 8 * e;
+    o[0] = r * L * W;
+    o[1] = (yp + L * z) * L * W;
+    o[2] = (ym + L * z) * L * W;
+    o[3] = (y + L * zp) * L * W;
+    o[4] = r * L;
+    o[5] = (y + L * zm) * L * W;
+  }
+}
+
+// ---- phases of a tile: init_tables and publish_levels serve both kernels,
+// gather_tile and store_tile are the Gaussian kernel's (nibble tiles)
+
+// Site records (bond masks, site/step parts of Philox rounds 1-3); all
+// `nthreads` threads of the CTA help.
+template <int L>
+__device__ __forceinline__ void init_tables(const SweepArgs& a, SiteRec* recs, int tid, int nthreads) {
+  constexpr int N = L * L * L;
+  for (int n = tid; n < N; n += nthreads) {
+    recs[n] = site_record(L, n, a.jtab, (uint32_t)a.t, a);
+  }
+}
+
+// The parent (old slot) of new slot j, -1 past R~.
+__device__ __forceinline__ int parent_of(const SweepArgs& a, int j, int R_new) {
+  return j < R_new ? (a.fresh ? j : a.pop.parents[j]) : -1;
+}
+
+// Levels and histogram of the tile's slots (after count_levels and a barrier).
+template <int TJ>
+__device__ __forceinline__ void publish_levels(const SweepArgs& a, const int* ecnt, int tile0, int R_new, int tid,
+                                               int nthreads) {
+  const PopDev& P = a.pop;
+  uint32_t* hist = P.hist + (size_t)a.t * a.n_levels;
+  for (int i = tid; i < TJ; i += nthreads) {
+    const int j = tile0 + i;
+    if (j < R_new) {
+      const int k = ecnt[i];
+      P.levels[j] = k;
+      atomicAdd(&hist[k], 1u);
+    }
+  }
+}
+
+// ---- +-1 couplings: the bit-sliced sweep
+
+// Bits needed to hold 0..n.
+constexpr int bits_for(int n) { return n < 2 ? 1 : 1 + bits_for(n / 2); }
+
+// A word whose replicas the first two Philox blocks (bit planes 0..7) leave
+// undecided: its site n and word (n | word << 16), the undecided replicas, and
+// bits 0 and 1 of their unsatisfied-bond counts.
+struct __align__(16) Deferred {
+  uint32_t loc, eq, u0, u1;
+};
+constexpr int kQueueCap = 64;  // a warp queues at most 31 + 32 words before it finishes 32 of them
+
+template <int L, int W, int NT, int MB>
+struct BitShape {
+  static constexpr int N = L * L * L;
+  static constexpr int ROWS = L * L;
+  static constexpr int NP = NT / W;       // row partitions
+  static constexpr int TJ = 32 * W;       // replicas per tile
+  static constexpr int SLOTS = 33 * W;    // parents (padded by one per word), then level counts
+  static constexpr int CB = bits_for(3 * L * (ROWS / NP));  // bit planes of a thread's level counter
+  static constexpr size_t SMEM_TILE = (size_t)N * W * 4 + (size_t)N * sizeof(SiteRec) + (size_t)SLOTS * 4;
+  static constexpr size_t SMEM_QUEUES = (size_t)(NT / 32) * kQueueCap * sizeof(Deferred);
+  static constexpr int RPP = ROWS / NP;  // rows per partition
+  static constexpr size_t SMEM_ROWS = (size_t)NP * RPP * 8 * sizeof(int);
+  // Deferred comparisons need whole warps that each stay inside one parity class
+  // (every lane of a warp then runs the same half-sweep code in step), and room
+  // for the queues without fewer than MB CTAs per SM (228 KB per SM, 1 KB of it
+  // reserved per CTA).
+  static constexpr bool DEFER = NT % 32 == 0 && ((NP / 2) * W) % 32 == 0 &&
+                                (size_t)MB * (SMEM_TILE + SMEM_QUEUES + SMEM_ROWS + 1024) <= 233472;
+  static constexpr int NQ = DEFER ? NT / 32 : 0;  // one queue per warp
+  static constexpr size_t SMEM = SMEM_TILE + (DEFER ? SMEM_QUEUES + SMEM_ROWS : 0);
+  static_assert(NT % W == 0 && 32 % W == 0 && NT <= 1024, "threads must tile the words of a row");
+  static_assert(L % 2 == 0 && L / 2 <= 8, "even L up to 16");
+  static_assert(NP % 2 == 0 && (ROWS / 2) % (NP / 2) == 0, "row partitions must split each parity class");
+  static_assert(1024 % TJ == 0, "a tile never crosses the 1024-slot pitch unit");
+};
+
+// One half-sweep of the rows of partition `part` (parity class p, colour sites at
+// x = X0 mod 2).  spw points at this thread's word of site 0; tp[b] are the
+// thread's hoisted Philox parts of block b for this half-sweep q; g8 = 8 x the
+// thread's global word index (the group of block b is g8 + b).
+template <int L, int W, int NP, int X0>
+__device__ __forceinline__ void sweep_rows_bits(uint32_t* spw, const SiteRec* recs, int part, int p,
+                                                const ThreadPhilox (&tp)[4], uint32_t q, uint32_t g8,
+                                                const SweepArgs& a) {
+  constexpr int H = L / 2, RPP = L * L / NP;
+#pragma unroll 1
+  for (int k = 0; k < RPP; ++k) {
+    const int r = row_index<L, NP>(part, k, p);
+    const int y = r % L, z = r / L;
+    const int yp = y == L - 1 ? 0 : y + 1, ym = y == 0 ? L - 1 : y - 1;
+    const int zp = z == L - 1 ? 0 : z + 1, zm = z == 0 ? L - 1 : z - 1;
+    uint32_t* p0 = spw + (size_t)r * L * W;
+    const uint32_t* pyp = spw + (size_t)(yp + L * z) * L * W;
+    const uint32_t* pym = spw + (size_t)(ym + L * z) * L * W;
+    const uint32_t* pzp = spw + (size_t)(y + L * zp) * L * W;
+    const uint32_t* pzm = spw + (size_t)(y + L * zm) * L * W;
+    const SiteRec* rr = recs + r * L;
+    const uint32_t h0 = (uint32_t)(r * L) >> 1;
+#pragma unroll 2  // two sites in flight: measured 3 % faster than one, as fast as all
+    for (int xh = 0; xh < H; ++xh) {
+      const int x = 2 * xh + X0;
+      const int xp = x == L - 1 ? 0 : x + 1, xm = x == 0 ? L - 1 : x - 1;
+      const SiteRec sr = rr[x];
+      const uint32_t s0 = p0[x * W];
+      // unsatisfied bonds (one bit per replica) and their count u in three planes
+      const uint32_t b0 = s0 ^ p0[xp * W] ^ sr.jxp, b1 = s0 ^ p0[xm * W] ^ sr.jxm;
+      const uint32_t b2 = s0 ^ pyp[x * W] ^ sr.jyp, b3 = s0 ^ pym[x * W] ^ sr.jym;
+      const uint32_t b4 = s0 ^ pzp[x * W] ^ sr.jzp, b5 = s0 ^ pzm[x * W] ^ sr.jzm;
+      const uint32_t sa = b0 ^ b1 ^ b2, ca = majority(b0, b1, b2);
+      const uint32_t sb = b3 ^ b4 ^ b5, cb = majority(b3, b4, b5);
+      const uint32_t u0 = sa ^ sb, k2 = sa & sb;
+      const uint32_t u1 = ca ^ cb ^ k2, u2 = majority(ca, cb, k2);
+      const uint32_t always = u2 | (u1 & u0);  // u >= 3: dE <= 0
+      // replicas to compare: u = 0, 1, 2 (dE = 12, 8, 4) with thr(u) > 0
+      uint32_t eq = ~always & threshold_bits(a.live, u0, u1);
+      uint32_t acc = 0;
+      const uint32_t uc = kM0 * (h0 + (uint32_t)xh);  // lo(M0 h), h = n >> 1
+      {
+        uint32_t w0[4], w1[4];
+        philox_block(uc, sr, tp[0], a.k0, a.k1, w0);
+        philox_block(uc, sr, tp[1], a.k0, a.k1, w1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) compare_plane(w0[i], u0, u1, a.tm[i], eq, acc);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) compare_plane(w1[i], u0, u1, a.tm[4 + i], eq, acc);
+      }
+      if (eq) {
+        uint32_t w[4];
+        philox_block(uc, sr, tp[2], a.k0, a.k1, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) compare_plane(w[i], u0, u1, a.tm[8 + i], eq, acc);
+      }
+      if (eq) {
+        uint32_t w[4];
+        philox_block(uc, sr, tp[3], a.k0, a.k1, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) compare_plane(w[i], u0, u1, a.tm[12 + i], eq, acc);
+      }
+#pragma unroll 1
+      for (int b = 4; b < 8 && eq; ++b) {  // rare: some replica matched its threshold for 16 bits
+        const ThreadPhilox tb = thread_philox(g8 + (uint32_t)b, q, a.k0, a.k1);
+        uint32_t w[4];
+        philox_block(uc, sr, tb, a.k0, a.k1, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) compare_plane(w[i], u0, u1, a.tm[4 * b + i], eq, acc);
+      }
+      p0[x * W] = s0 ^ (acc | always);
+    }
+  }
+}
+
+// Finishes a deferred word: Philox blocks 2, 3, ... of its site and group until
+// every queued replica is decided, then flips the accepted ones (the word's owner
+// has already applied the flips decided in planes 0..7).  Any lane of the owner's
+// warp may run it: the same-colour sites of a half-sweep are independent.
+template <int W>
+__device__ __forceinline__ void finish_deferred(uint32_t* sp, const SiteRec* recs, const Deferred d, uint32_t q,
+                                                uint32_t gbase, const SweepArgs& a) {
+  const int n = (int)(d.loc & 0xffffu), word = (int)(d.loc >> 16);
+  sp[n * W + word] ^=
+      compare_rest(d.eq, d.u0, d.u1, (uint32_t)n, recs[n], 8u * (gbase + (uint32_t)word), q, a);
+}
+
+// One half-sweep of the rows of partition `part`, as sweep_rows_bits, for shapes
+// whose warps stay inside one parity class: a word still undecided after blocks
+// 0 and 1 (about one in eight) goes to the warp's queue dq, and whenever 32 are
+// queued the warp finishes them with all lanes (finish_deferred); the rest are
+// finished at the end of the half-sweep.  The decisions are the same; only the
+// lanes that take them change.  sp: the tile (word-major within a site row);
+// gbase: the tile's first word index (Philox group 8 (gbase + word) + b); rowtab:
+// per partition and row the word offsets of the row and its four neighbour rows
+// and the row's first site (built once per tile: a thread's rows never change).
+// The sites of a row are unrolled, so every column offset is a constant.
+template <int L, int W, int NP, int X0, int FORM>
+__device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const SiteRec* recs, int part, int p,
+                                                   const ThreadPhilox (&tp)[2], uint32_t q, uint32_t gbase,
+                                                   Deferred* dq, const int* rowtab, const SweepArgs& a) {
+  constexpr int H = L / 2, RPP = L * L / NP;
+  const int lane = (int)(threadIdx.x & 31u);
+  const unsigned below = (1u << lane) - 1u;
+  uint32_t* spw = sp + word;
+  int head = 0, cnt = 0;  // the same in every lane of the warp
+#pragma unroll 1
+  for (int k = 0; k < RPP; ++k) {
+    const int4 e0 = *reinterpret_cast<const int4*>(rowtab + 8 * (part * RPP + k));
+    const int rL = rowtab[8 * (part * RPP + k) + 4];
+    uint32_t* p0 = spw + e0.x;
+    const uint32_t* pyp = spw + e0.y;
+    const uint32_t* pym = spw + e0.z;
+    const uint32_t* pzp = spw + e0.w;
+    const uint32_t* pzm = spw + rowtab[8 * (part * RPP + k) + 5];
+    const SiteRec* rr = recs + rL;
+    const uint32_t h0 = (uint32_t)rL >> 1;
+#pragma unroll
+    for (int xh = 0; xh < H; ++xh) {
+      const int x = 2 * xh + X0;
+      const int xp = x == L - 1 ? 0 : x + 1, xm = x == 0 ? L - 1 : x - 1;
+      const SiteRec sr = rr[x];
+      const uint32_t s0 = p0[x * W];
+      const BondCount c = bond_count(s0, sr, p0[xp * W], p0[xm * W], pyp[x * W], pym[x * W], pzp[x * W], pzm[x * W], a);
+      uint32_t lt, eq;
+      compare_planes8<FORM>(kM0 * (h0 + (uint32_t)xh), sr, tp, c, a, lt, eq);  // lo(M0 h), h = n >> 1
+      p0[x * W] = s0 ^ (lt | c.always);
+      const unsigned dm = __ballot_sync(0xffffffffu, eq != 0u);
+      if (eq) {
+        Deferred d;
+        d.loc = (uint32_t)(rL + x) | ((uint32_t)word << 16);
+        d.eq = eq;
+        d.u0 = c.u0;
+        d.u1 = c.u1;
+        dq[(head + cnt + __popc(dm & below)) & (kQueueCap - 1)] = d;
+      }
+      cnt += __popc(dm);
+      if (cnt >= 32) {
+        __syncwarp();
+        finish_deferred<W>(sp, recs, dq[(head + lane) & (kQueueCap - 1)], q, gbase, a);
+        __syncwarp();
+        head = (head + 32) & (kQueueCap - 1);
+        cnt -= 32;
+      }
+    }
+  }
+  __syncwarp();
+  if (lane < cnt) finish_deferred<W>(sp, recs, dq[(head + lane) & (kQueueCap - 1)], q, gbase, a);
+  __syncwarp();
+}
+
+// Gather the tile's spins from the parents of its slots into bit words; spar
+// holds the tile's parents (-1 past R~), slot i at index 33 (i >> 5) + (i & 31).
+// A thread takes 32 slots (one word of the tile) and BW words of their rows, 32 BW
+// sites: BW loads of each row, a transpose, 32 BW words of the tile.  Consecutive
+// threads take consecutive words of a site row, so the shared-memory stores have no
+// bank conflicts; the rows are read in pieces of 4 BW bytes, a sector's other pieces
+// by other warps at the same time (L1).  BW = 2 where 64 words fit the registers.
+template <int L, int W, int NT, int MB>
+struct RowMove : Row<L> {
+  using Row<L>::SW;
+  using Row<L>::NB;
+  static constexpr int BW = SW % 2 == 0 && NT * MB <= 640 ? 2 : 1;
+  static constexpr int GATHER_UNITS = W * ((NB + BW - 1) / BW);
+  static constexpr int STORE_UNITS = W * (SW / BW);  // the padding of a row too: its bits stay 0
+};
+
+template <int L, int W, int NT, int MB>
+__device__ __forceinline__ void gather_bits(const SweepArgs& a, uint32_t* sp, const int* spar) {
+  using M = RowMove<L, W, NT, MB>;
+  const uint32_t* src = a.pop.spins[a.cur];
+  for (int u = threadIdx.x; u < M::GATHER_UNITS; u += NT) {
+    const int word = u % W, blk = u / W * M::BW;
+    uint32_t m[M::BW][32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      const int p = spar[33 * word + i];
+      const uint32_t* row = src + (size_t)(p >= 0 ? p : 0) * M::SW + blk;
+      if constexpr (M::BW == 2) {
+        const uint2 v = p >= 0 ? *reinterpret_cast<const uint2*>(row) : make_uint2(0u, 0u);
+        m[0][i] = v.x;
+        m[1][i] = v.y;
+      } else {
+        m[0][i] = p >= 0 ? *row : 0u;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < M::BW; ++h) {
+      transpose32(m[h]);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int n = 32 * (blk + h) + i;
+        if (M::N % (32 * M::BW) == 0 || n < M::N) sp[n * W + word] = m[h][i];
+      }
+    }
+  }
+}
+
+// Unsatisfied forward bonds of every replica of the tile, counted per thread in
+// CB bit planes and then added per replica into ecnt (slot i at index i).
+template <int L, int W, int NP, int CB>
+__device__ __forceinline__ void count_levels_bits(const uint32_t* sp, const SiteRec* recs, int* ecnt, int word,
+                                                  int part) {
+  constexpr int ROWS = L * L;
+  uint32_t c[CB];
+#pragma unroll
+  for (int i = 0; i < CB; ++i) c[i] = 0;
+  for (int r = part; r < ROWS; r += NP) {
+    const int y = r % L, z = r / L;
+    const int yp = y == L - 1 ? 0 : y + 1, zp = z == L - 1 ? 0 : z + 1;
+    const uint32_t* p0 = sp + (size_t)r * L * W + word;
+    const uint32_t* pyp = sp + (size_t)(yp + L * z) * L * W + word;
+    const uint32_t* pzp = sp + (size_t)(y + L * zp) * L * W + word;
+    const SiteRec* rr = recs + r * L;
+#pragma unroll
+    for (int x = 0; x < L; ++x) {
+      const int xp = x == L - 1 ? 0 : x + 1;
+      const uint32_t s0 = p0[x * W];
+      const uint32_t e0 = s0 ^ p0[xp * W] ^ rr[x].jxp, e1 = s0 ^ pyp[x * W] ^ rr[x].jyp,
+                     e2 = s0 ^ pzp[x * W] ^ rr[x].jzp;
+      const uint32_t sum = e0 ^ e1 ^ e2, two = majority(e0, e1, e2);  // e0 + e1 + e2 = sum + 2 two
+      uint32_t carry = c[0] & sum;
+      c[0] ^= sum;
+      const uint32_t c1 = c[1] ^ two ^ carry;
+      carry = majority(c[1], two, carry);
+      c[1] = c1;
+#pragma unroll
+      for (int i = 2; i < CB; ++i) {
+        const uint32_t ci = c[i] ^ carry;
+        carry &= c[i];
+        c[i] = ci;
+      }
+    }
+  }
+#pragma unroll 1
+  for (int bb = 0; bb < 32; ++bb) {
+    const int b = (bb + word) & 31;  // lanes of a warp hit different banks
+    int k = 0;
+#pragma unroll
+    for (int i = 0; i < CB; ++i) k |= (int)((c[i] >> b) & 1u) << i;
+    if (k) atomicAdd(&ecnt[32 * word + b], k);
+  }
+}
+
+// Write the tile back to the rows of its slots, the gather's split reversed.
+template <int L, int W, int NT, int MB>
+__device__ __forceinline__ void store_bits(const SweepArgs& a, const uint32_t* sp, int tile0) {
+  using M = RowMove<L, W, NT, MB>;
+  uint32_t* dst = a.pop.spins[1 - a.cur];
+  for (int u = threadIdx.x; u < M::STORE_UNITS; u += NT) {
+    const int word = u % W, blk = u / W * M::BW;
+    uint32_t m[M::BW][32];
+#pragma unroll
+    for (int h = 0; h < M::BW; ++h) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int n = 32 * (blk + h) + i;
+        m[h][i] = n < M::N ? sp[n * W + word] : 0u;
+      }
+      transpose32(m[h]);
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      uint32_t* row = dst + (size_t)(tile0 + 32 * word + i) * M::SW + blk;
+      if constexpr (M::BW == 2)
+        *reinterpret_cast<uint2*>(row) = make_uint2(m[0][i], m[1][i]);
+      else
+        *row = m[0][i];
+    }
+  }
+}
+
+// Families (a7) of the tile's new slots, so that a step needs no family launch
+// of its own: a family is a run of equal labels along the slots (labels ascend).
+// sh (shared memory, free by now) holds labs[0..TJ] (the slot before the tile,
+// then the tile's slots; -1 past R~), a bit mask per 32 slots of the slots that
+// start a run, and 64 words for the final sum.  The thread at a run's first slot
+// takes its end from the next start in the tile, or, for the tile's last run, by
+// galloping through the labels after the tile (run_end), and records the family
+// (pa_family.cuh); the last tile to finish adds the entropy.
+template <int TJ, int NT>
+__device__ __forceinline__ void tile_families(const SweepArgs& a, int* sh, int tile0, int R_new, int tid) {
+  constexpr int NC = TJ / 32;  // chunks of 32 slots (TJ <= 1024)
+  static_assert(NT % 32 == 0 || TJ <= NT, "the lanes of a warp take whole chunks");
+  int* labs = sh;
+  unsigned* bm = reinterpret_cast<unsigned*>(sh + TJ + 1);  // [NC + 1]: start bits per chunk, then chunks with starts
+  long long* red = reinterpret_cast<long long*>(sh + ((TJ + 1 + NC + 2) & ~1));
+  const int32_t* lab = a.pop.labels[1 - a.cur];
+  const unsigned mask = warp_lanes(tid, NT);
+  for (int i = tid; i <= TJ; i += NT) {
+    const int j = tile0 - 1 + i;
+    labs[i] = (j >= 0 && j < R_new) ? lab[j] : -1;
+  }
+  __syncthreads();
+  // run starts, one ballot per chunk (lanes of a warp take consecutive slots)
+  for (int base = 0; base < TJ; base += NT) {
+    const int i = base + tid;
+    const bool start = i < TJ && labs[i + 1] != labs[i];
+    const unsigned b = __ballot_sync(mask, start);
+    if ((i & 31) == 0 && i < TJ) bm[i >> 5] = b;
+  }
+  __syncthreads();
+  if (tid < 32) {  // chunks that hold a run start
+    const unsigned nzb = __ballot_sync(0xffffffffu, tid < NC && bm[tid] != 0u);
+    if (tid == 0) bm[NC] = nzb;
+  }
+  __syncthreads();
+  const unsigned nz = bm[NC];
+  FamilyAcc f;
+  for (int base = 0; base < TJ; base += NT) {  // the same iterations in every lane of a warp
+    const int i = base + tid, j = tile0 + i, c = i >> 5, l = i & 31;
+    int eta = 0;
+    if (i < TJ && j < R_new && (bm[c] >> l & 1u)) {
+      const unsigned above = l == 31 ? 0u : bm[c] & (~0u << (l + 1));
+      const unsigned later = c == 31 ? 0u : nz & (~0u << (c + 1));
+      int end;
+      if (above) {
+        end = tile0 + 32 * c + __ffs(above) - 1;
+      } else if (later) {
+        const int c2 = __ffs(later) - 1;
+        end = tile0 + 32 * c2 + __ffs(bm[c2]) - 1;
+      } else {
+        end = run_end(lab, labs[i + 1], tile0 + TJ, R_new);
+      }
+      eta = end - j;
+      f.add(eta);
+    }
+    family_size(a.pop, eta, mask);
+  }
+  family_flush(f, mask, &a.pop.rec[a.t]);
+  // the tiles of both launches that hold slots take part
+  const int in_main = min(R_new, a.split);
+  const int participants = (in_main + a.tj_main - 1) / a.tj_main +
+                           (R_new > a.split ? (R_new - a.split + a.tj_tail - 1) / a.tj_tail : 0);
+  family_entropy_last(a.pop, &a.pop.rec[a.t], R_new, participants, tid, NT, red);
+}
+
+template <int F>
+struct Form {
+  static constexpr int value = F;
+};
+
+// One tile of the bit-sliced sweep (+-1 couplings): the slots tile0 .. tile0 + TJ - 1
+// of the new population (R_new slots), in the dynamic shared memory sm.
+template <int L, int W, int NT, int MB>
+__device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int tile0, int R_new) {
+  using S = BitShape<L, W, NT, MB>;
+  constexpr int N = S::N, NP = S::NP, TJ = S::TJ;
+  uint32_t* sp = sm;                                               // spins [N][W]
+  SiteRec* recs = reinterpret_cast<SiteRec*>(sm + (size_t)N * W);  // [N]
+  Deferred* queues = reinterpret_cast<Deferred*>(recs + N);        // [NQ][kQueueCap]
+  int* slots = reinterpret_cast<int*>(queues + S::NQ * kQueueCap);  // [33 W]: parents, then level counts
+  int* rowtab = slots + S::SLOTS;  // [NP][RPP][8]: word offsets of a row and its four neighbour rows, its first site
+  const int tid = threadIdx.x, word = tid % W, part = tid / W;
+  Deferred* dq = queues + (S::DEFER ? (tid >> 5) * kQueueCap : 0);
+  init_tables<L>(a, recs, tid, NT);
+  if constexpr (S::DEFER) fill_row_table<L, W, NP>(rowtab, tid, NT);
+  for (int i = tid; i < TJ; i += NT) slots[33 * (i >> 5) + (i & 31)] = parent_of(a, tile0 + i, R_new);
+  __syncthreads();
+  gather_bits<L, W, NT, MB>(a, sp, slots);
+  __syncthreads();
+  for (int i = tid; i < S::SLOTS; i += NT) slots[i] = 0;
+  __syncthreads();
+
+  // sweeps: partition `part` owns rows of parity class p = (y + z) & 1; in
+  // half-sweep c its colour sites sit at x = p ^ c mod 2 in every row.
+  const uint32_t gbase = (uint32_t)((a.slot_base + tile0) >> 5);  // global index of the tile's first word
+  const uint32_t g8 = 8u * (gbase + (uint32_t)word);             // Philox group of block 0 of this word
+  const int pclass = part / (NP / 2);
+  if constexpr (S::DEFER) {
+    auto sweeps = [&](auto form) {
+      constexpr int FORM = decltype(form)::value;
+      for (uint32_t q = 0; q < 2u * (uint32_t)a.n_sweeps; ++q) {
+        const ThreadPhilox tp[2] = {thread_philox(g8, q, a.k0, a.k1), thread_philox(g8 + 1u, q, a.k0, a.k1)};
+        if ((pclass ^ (int)(q & 1u)) == 0)  // the same in every lane of the warp
+          sweep_rows_bits_dq<L, W, NP, 0, FORM>(sp, word, recs, part, pclass, tp, q, gbase, dq, rowtab, a);
+        else
+          sweep_rows_bits_dq<L, W, NP, 1, FORM>(sp, word, recs, part, pclass, tp, q, gbase, dq, rowtab, a);
+        __syncthreads();
+      }
+    };
+    switch (a.form) {  // the same in every thread: the step's thresholds decide
+      case 3: sweeps(Form<3>{}); break;
+      case 2: sweeps(Form<2>{}); break;
+      case 1: sweeps(Form<1>{}); break;
+      default: sweeps(Form<0>{}); break;
+    }
+  } else {
+    uint32_t* spw = sp + word;
+#pragma unroll 1
+    for (uint32_t q = 0; q < 2u * (uint32_t)a.n_sweeps; ++q) {
+      const ThreadPhilox tp[4] = {thread_philox(g8, q, a.k0, a.k1), thread_philox(g8 + 1u, q, a.k0, a.k1),
+                                  thread_philox(g8 + 2u, q, a.k0, a.k1), thread_philox(g8 + 3u, q, a.k0, a.k1)};
+      if ((pclass ^ (int)(q & 1u)) == 0)
+        sweep_rows_bits<L, W, NP, 0>(spw, recs, part, pclass, tp, q, g8, a);
+      else
+        sweep_rows_bits<L, W, NP, 1>(spw, recs, part, pclass, tp, q, g8, a);
+      __syncthreads();
+    }
+  }
+  count_levels_bits<L, W, NP, S::CB>(sp, recs, slots, word, part);
+  __syncthreads();
+  publish_levels<TJ>(a, slots, tile0, R_new, tid, NT);
+  store_bits<L, W, NT, MB>(a, sp, tile0);
+  if (!a.fam) return;
+  __syncthreads();  // every shared array is dead now: the family pass takes the space
+  tile_families<TJ, NT>(a, reinterpret_cast<int*>(sm), tile0, R_new, tid);
+}
+
+// Bit-sliced sweep kernel (+-1 couplings): one tile per CTA.
+template <int L, int W, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) k_sweep(const __grid_constant__ SweepArgs a) {
+  extern __shared__ __align__(16) uint32_t sm[];
+  const int R_new = a.pop.rec[a.t].R_tilde;
+  const int tile0 = a.tile_base + blockIdx.x * BitShape<L, W, NT, MB>::TJ;
+  if (tile0 >= R_new) return;
+  sweep_tile<L, W, NT, MB>(a, sm, tile0, R_new);
+}
+
+// The sweep arguments of population P at step t from buffer cur with thresholds
+// thr (dE = 4, 8, 12), as launch_sweep sets them for a run of one launch.
+__host__ __device__ inline void fill_sweep_args(SweepArgs& a, const PopDev& P, const uint32_t* jtab,
+                                                int n_levels, int t, int cur, int n_sweeps, int tj,
+                                                const uint32_t thr[3]) {
+  a.pop = P;
+  fill_metropolis(a, P.key_met, thr);
+  a.jtab = jtab;
+  a.n_levels = n_levels;
+  a.t = t;
+  a.cur = cur;
+  a.n_sweeps = n_sweeps;
+  a.slot_base = 0;
+  a.fam = 1;
+  a.fresh = 0;
+  a.tile_base = 0;
+  a.split = 0x7fffffff;
+  a.tj_main = tj;
+  a.tj_tail = tj;
+}
+
+// The sweeps of a batch's units of one lattice size and launch shape: unit list[k]
+// takes the CTAs off[k] .. off[k+1]-1, one tile each; each CTA builds its unit's
+// arguments for the round's step in shared memory.
+template <int L, int W, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB)
+    k_sweep_group(const GroupUnit* __restrict__ units, const int32_t* __restrict__ list,
+                  const int32_t* __restrict__ off, int n, const int32_t* __restrict__ round) {
+  constexpr int TJ = BitShape<L, W, NT, MB>::TJ;
+  extern __shared__ __align__(16) uint32_t sm[];
+  __shared__ SweepArgs sa;
+  __shared__ int hdr[3];  // unit, tile0, R_new (tile0 < 0: nothing to do)
+  if (threadIdx.x == 0) {
+    int lo = 0, hi = n - 1;
+    const int b = (int)blockIdx.x;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (off[mid] <= b) lo = mid; else hi = mid - 1;
+    }
+    const GroupUnit& u = units[list[lo]];
+    const int r = *round, t = u.t0 + 1 + r;
+    const int tile0 = (b - off[lo]) * TJ;
+    const int R_new = t <= u.last_t ? u.P.rec[t].R_tilde : 0;
+    hdr[0] = list[lo];
+    hdr[1] = tile0 < R_new ? tile0 : -1;
+    hdr[2] = R_new;
+    if (tile0 < R_new) {
+      const GroupStep& st = u.steps[t];
+      fill_sweep_args(sa, u.P, u.jtab, u.g.n_levels, t, u.cur0 ^ (r & 1), st.n_sweeps, TJ, st.thr);
+    }
+  }
+  __syncthreads();
+  if (hdr[1] < 0) return;
+  sweep_tile<L, W, NT, MB>(sa, sm, hdr[1], hdr[2]);
+}
+
+template <int L, int W, int NT, int MB>
+static int launch_group_t(const GroupUnit* units, const int32_t* list, const int32_t* off, int n, int n_blocks,
+                          const int32_t* round, cudaStream_t s) {
+  using S = BitShape<L, W, NT, MB>;
+  static std::atomic<int> done[64];
+  const cudaError_t e = smem_limit_once(k_sweep_group<L, W, NT, MB>, (int)S::SMEM, done);
+  if (e != cudaSuccess) return (int)e;
+  if (n_blocks <= 0) return 0;
+  k_sweep_group<L, W, NT, MB><<<n_blocks, NT, S::SMEM, s>>>(units, list, off, n, round);
+  return (int)cudaGetLastError();
+}
+
+template <int L, int W, int NT, int MB>
+static int launch_t(const RunGeom& g, const SweepArgs& args, cudaStream_t s) {
+  using S = BitShape<L, W, NT, MB>;
+  static std::atomic<int> done[64];
+  const cudaError_t e = smem_limit_once(k_sweep<L, W, NT, MB>, (int)S::SMEM, done);
+  if (e != cudaSuccess) return (int)e;
+  // tiles from tile_base up to the split (main launch) or to the capacity (tail launch)
+  const int64_t end = args.tile_base < args.split ? std::min<int64_t>(args.split, g.R_cap) : g.R_cap;
+  if (end <= args.tile_base) return 0;
+  dim3 grid((unsigned)((end - args.tile_base + S::TJ - 1) / S::TJ));
+  k_sweep<L, W, NT, MB><<<grid, NT, S::SMEM, s>>>(args);
+  return (int)cudaGetLastError();
+}
+
+// One launch shape of the +-1 sweep.
+struct ShapeEntry {
+  int L, W, NT, MB;
+  size_t smem;
+  int (*launch)(const RunGeom&, const SweepArgs&, cudaStream_t);
+  int (*launch_group)(const GroupUnit*, const int32_t*, const int32_t*, int, int, const int32_t*, cudaStream_t);
+};
+#define PA_SHAPE(L, W, NT, MB) \
+  {L, W, NT, MB, BitShape<L, W, NT, MB>::SMEM, &launch_t<L, W, NT, MB>, &launch_group_t<L, W, NT, MB>}
+
+// The shapes of one lattice size, default first.
+struct ShapeList {
+  const ShapeEntry* e;
+  int n;
+};
+ShapeList sweep_shapes_2();
+ShapeList sweep_shapes_4();
+ShapeList sweep_shapes_6();
+ShapeList sweep_shapes_8();
+ShapeList sweep_shapes_10();
+ShapeList sweep_shapes_12();
+ShapeList sweep_shapes_14();
+ShapeList sweep_shapes_16();
+
+}  // namespace pa
