@@ -118,22 +118,6 @@ __device__ __forceinline__ int parent_of(const SweepArgs& a, int j, int R_new) {
   return j < R_new ? (a.fresh ? j : a.pop.parents[j]) : -1;
 }
 
-// Levels and histogram of the tile's slots (after count_levels and a barrier).
-template <int TJ>
-__device__ __forceinline__ void publish_levels(const SweepArgs& a, const int* ecnt, int tile0, int R_new, int tid,
-                                               int nthreads) {
-  const PopDev& P = a.pop;
-  uint32_t* hist = P.hist + (size_t)a.t * a.n_levels;
-  for (int i = tid; i < TJ; i += nthreads) {
-    const int j = tile0 + i;
-    if (j < R_new) {
-      const int k = ecnt[i];
-      P.levels[j] = k;
-      atomicAdd(&hist[k], 1u);
-    }
-  }
-}
-
 // ---- +-1 couplings: the bit-sliced sweep
 
 // Bits needed to hold 0..n.
@@ -145,7 +129,7 @@ constexpr int bits_for(int n) { return n < 2 ? 1 : 1 + bits_for(n / 2); }
 struct __align__(16) Deferred {
   uint32_t loc, eq, u0, u1;
 };
-constexpr int kQueueCap = 64;  // a warp queues at most 31 + 32 words before it finishes 32 of them
+constexpr int kQueueCap = 64;  // words a warp queues; it finishes 32 of them as soon as there are
 
 template <int L, int W, int NT, int MB>
 struct BitShape {
@@ -269,7 +253,12 @@ __device__ __forceinline__ void finish_deferred(uint32_t* sp, const SiteRec* rec
 // gbase: the tile's first word index (Philox group 8 (gbase + word) + b); rowtab:
 // per partition and row the word offsets of the row and its four neighbour rows
 // and the row's first site (built once per tile: a thread's rows never change).
-// The sites of a row are unrolled, so every column offset is a constant.
+//
+// The sites of a row are unrolled, so every column offset is a constant, and form one
+// straight piece of code: the row's spins stay in registers, its new words are stored
+// and its undecided words queued after the last site.  The multiplies of one site's
+// Philox blocks (the FMA pipe, 32 wide products of 4 cycles each per warp) then run
+// beside the logic of another's (the ALU pipe, 2 cycles per operation).
 template <int L, int W, int NP, int X0, int FORM>
 __device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const SiteRec* recs, int part, int p,
                                                    const ThreadPhilox (&tp)[2], uint32_t q, uint32_t gbase,
@@ -279,6 +268,19 @@ __device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const
   const unsigned below = (1u << lane) - 1u;
   uint32_t* spw = sp + word;
   int head = 0, cnt = 0;  // the same in every lane of the warp
+  auto push = [&](int n, uint32_t eq, const BondCount& c, unsigned dm) {
+    if (eq) dq[(head + cnt + __popc(dm & below)) & (kQueueCap - 1)] =
+        Deferred{(uint32_t)n | ((uint32_t)word << 16), eq, c.u0, c.u1};
+    cnt += __popc(dm);
+  };
+  auto finish = [&]() {  // the 32 oldest, or all there are
+    __syncwarp();
+    if (lane < cnt) finish_deferred<W>(sp, recs, dq[(head + lane) & (kQueueCap - 1)], q, gbase, a);
+    __syncwarp();
+    const int done = min(cnt, 32);
+    head = (head + done) & (kQueueCap - 1);
+    cnt -= done;
+  };
 #pragma unroll 1
   for (int k = 0; k < RPP; ++k) {
     const int4 e0 = *reinterpret_cast<const int4*>(rowtab + 8 * (part * RPP + k));
@@ -290,96 +292,169 @@ __device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const
     const uint32_t* pzm = spw + rowtab[8 * (part * RPP + k) + 5];
     const SiteRec* rr = recs + rL;
     const uint32_t h0 = (uint32_t)rL >> 1;
+    uint32_t row[L];
+#pragma unroll
+    for (int x = 0; x < L; ++x) row[x] = p0[x * W];
+    uint32_t eq[H];
+    BondCount c[H];
 #pragma unroll
     for (int xh = 0; xh < H; ++xh) {
       const int x = 2 * xh + X0;
       const int xp = x == L - 1 ? 0 : x + 1, xm = x == 0 ? L - 1 : x - 1;
       const SiteRec sr = rr[x];
-      const uint32_t s0 = p0[x * W];
-      const BondCount c = bond_count(s0, sr, p0[xp * W], p0[xm * W], pyp[x * W], pym[x * W], pzp[x * W], pzm[x * W], a);
-      uint32_t lt, eq;
-      compare_planes8<FORM>(kM0 * (h0 + (uint32_t)xh), sr, tp, c, a, lt, eq);  // lo(M0 h), h = n >> 1
-      p0[x * W] = s0 ^ (lt | c.always);
-      const unsigned dm = __ballot_sync(0xffffffffu, eq != 0u);
-      if (eq) {
-        Deferred d;
-        d.loc = (uint32_t)(rL + x) | ((uint32_t)word << 16);
-        d.eq = eq;
-        d.u0 = c.u0;
-        d.u1 = c.u1;
-        dq[(head + cnt + __popc(dm & below)) & (kQueueCap - 1)] = d;
-      }
-      cnt += __popc(dm);
-      if (cnt >= 32) {
-        __syncwarp();
-        finish_deferred<W>(sp, recs, dq[(head + lane) & (kQueueCap - 1)], q, gbase, a);
-        __syncwarp();
-        head = (head + 32) & (kQueueCap - 1);
-        cnt -= 32;
+      c[xh] = bond_count(row[x], sr, row[xp], row[xm], pyp[x * W], pym[x * W], pzp[x * W], pzm[x * W], a);
+      uint32_t lt;
+      compare_planes8<FORM>(kM0 * (h0 + (uint32_t)xh), sr, tp, c[xh], a, lt, eq[xh]);  // lo(M0 h), h = n >> 1
+      row[x] ^= lt | c[xh].always;
+    }
+#pragma unroll
+    for (int xh = 0; xh < H; ++xh) p0[(2 * xh + X0) * W] = row[2 * xh + X0];
+    unsigned dm[H];
+    int total = cnt;
+#pragma unroll
+    for (int xh = 0; xh < H; ++xh) {
+      dm[xh] = __ballot_sync(0xffffffffu, eq[xh] != 0u);
+      total += __popc(dm[xh]);
+    }
+    if (total <= kQueueCap) {
+#pragma unroll
+      for (int xh = 0; xh < H; ++xh) push(rL + 2 * xh + X0, eq[xh], c[xh], dm[xh]);
+    } else {  // the row does not fit beside what is queued: room for each site's words first
+#pragma unroll
+      for (int xh = 0; xh < H; ++xh) {
+        while (cnt > kQueueCap - 32) finish();
+        push(rL + 2 * xh + X0, eq[xh], c[xh], dm[xh]);
       }
     }
+    while (cnt >= 32) finish();
   }
-  __syncwarp();
-  if (lane < cnt) finish_deferred<W>(sp, recs, dq[(head + lane) & (kQueueCap - 1)], q, gbase, a);
-  __syncwarp();
+  finish();
 }
 
-// Gather the tile's spins from the parents of its slots into bit words; spar
-// holds the tile's parents (-1 past R~), slot i at index 33 (i >> 5) + (i & 31).
-// A thread takes 32 slots (one word of the tile) and BW words of their rows, 32 BW
-// sites: BW loads of each row, a transpose, 32 BW words of the tile.  Consecutive
-// threads take consecutive words of a site row, so the shared-memory stores have no
-// bank conflicts; the rows are read in pieces of 4 BW bytes, a sector's other pieces
-// by other warps at the same time (L1).  BW = 2 where 64 words fit the registers.
+// How a shape moves its tile between the rows of its slots and its site-major words.
+// A thread transposes the 32 x 32 BW bits of 32 slots (a word column of the tile) and
+// BW words of their rows; BW = 2 where 64 words fit the registers.
+//
+// STAGED: the rows of the whole tile lie in shared memory in between, in place of the
+// tile's words (every thread holds its bits in registers while the layout changes, so
+// one pass must take the tile, and the rows must fit before the slot table).  The rows
+// then come in by 16-byte asynchronous copies, all in flight at once, and go out as
+// one bulk copy of contiguous memory.  Otherwise each thread reads and writes its
+// pieces of 4 BW bytes in global memory.  At L = 10 (1024 slots, 128 KB) the pieces
+// took 10.5 us to gather and 11 to 21 us to store.
 template <int L, int W, int NT, int MB>
 struct RowMove : Row<L> {
+  using S = BitShape<L, W, NT, MB>;
+  using Row<L>::N;
   using Row<L>::SW;
   using Row<L>::NB;
   static constexpr int BW = SW % 2 == 0 && NT * MB <= 640 ? 2 : 1;
   static constexpr int GATHER_UNITS = W * ((NB + BW - 1) / BW);
   static constexpr int STORE_UNITS = W * (SW / BW);  // the padding of a row too: its bits stay 0
+  static constexpr size_t SLOT_TABLE = (size_t)N * W * 4 + (size_t)N * sizeof(SiteRec) +
+                                       (size_t)S::NQ * kQueueCap * sizeof(Deferred);  // its offset in bytes
+  static constexpr int ROW_WORDS = 32 * W * SW;
+  static constexpr bool STAGED = STORE_UNITS <= NT && (size_t)ROW_WORDS * 4 <= SLOT_TABLE;
+  // Shared memory of the measurements after the store (level counts of the tile, then
+  // the families): behind the rows while they are copied out, or in their place.
+  static constexpr int LEVELS = 3 * N + 1;
+  static constexpr int FAM_WORDS = ((32 * W + 1 + W + 2) & ~1) + 128;
+  static constexpr int POST_WORDS = LEVELS > FAM_WORDS ? LEVELS : FAM_WORDS;
+  static constexpr bool POST_BEHIND = STAGED && (size_t)(ROW_WORDS + POST_WORDS) * 4 <= SLOT_TABLE;
+  static constexpr int POST = POST_BEHIND ? ROW_WORDS : 0;
 };
 
+// The unit's word column and first row word.  Neighbouring lanes take neighbouring
+// word columns, and (STAGED) row words one step apart, which spreads both the rows and
+// the words over the banks.
+template <typename M, int W, int UNITS>
+__device__ __forceinline__ void move_unit(int u, int& word, int& blk) {
+  constexpr int NBLK = UNITS / W;
+  word = u % W;
+  blk = (M::STAGED ? (u / W + word) % NBLK : u / W) * M::BW;
+}
+
+template <int BYTES>
+__device__ __forceinline__ void copy_async(uint32_t dst, const void* src, bool zero) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES),
+               "r"(zero ? 0 : BYTES)
+               : "memory");
+}
+
+// Gather the tile's spins from the parents of its slots into bit words; spar
+// holds the tile's parents (-1 past R~), slot i at index 33 (i >> 5) + (i & 31).
+// Ends with the words written but not yet synchronised; the site records may be
+// written from then on, not before (STAGED).
 template <int L, int W, int NT, int MB>
 __device__ __forceinline__ void gather_bits(const SweepArgs& a, uint32_t* sp, const int* spar) {
   using M = RowMove<L, W, NT, MB>;
   const uint32_t* src = a.pop.spins[a.cur];
-  for (int u = threadIdx.x; u < M::GATHER_UNITS; u += NT) {
-    const int word = u % W, blk = u / W * M::BW;
-    uint32_t m[M::BW][32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int p = spar[33 * word + i];
-      const uint32_t* row = src + (size_t)(p >= 0 ? p : 0) * M::SW + blk;
-      if constexpr (M::BW == 2) {
-        const uint2 v = p >= 0 ? *reinterpret_cast<const uint2*>(row) : make_uint2(0u, 0u);
-        m[0][i] = v.x;
-        m[1][i] = v.y;
-      } else {
-        m[0][i] = p >= 0 ? *row : 0u;
-      }
+  if constexpr (M::STAGED) {
+    constexpr int CW = M::SW % 4 == 0 ? 4 : M::SW;  // words per copy
+    constexpr int CPR = M::SW / CW;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(sp);
+    for (int e = threadIdx.x; e < 32 * W * CPR; e += NT) {
+      const int r = e / CPR, o = e % CPR * CW;
+      const int p = spar[33 * (r >> 5) + (r & 31)];
+      copy_async<4 * CW>(base + 4u * (uint32_t)(r * M::SW + o), src + (size_t)(p >= 0 ? p : 0) * M::SW + o, p < 0);
     }
-#pragma unroll
-    for (int h = 0; h < M::BW; ++h) {
-      transpose32(m[h]);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+  }
+  for (int u0 = 0; u0 < M::GATHER_UNITS; u0 += NT) {  // one pass when STAGED
+    const int u = u0 + threadIdx.x;
+    const bool on = u < M::GATHER_UNITS;
+    uint32_t m[M::BW][32];
+    int word = 0, blk = 0;
+    if (on) {
+      move_unit<M, W, M::GATHER_UNITS>(u, word, blk);
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
-        const int n = 32 * (blk + h) + i;
-        if (M::N % (32 * M::BW) == 0 || n < M::N) sp[n * W + word] = m[h][i];
+        const int p = M::STAGED ? 32 * word + i : spar[33 * word + i];
+        const uint32_t* row = (M::STAGED ? sp : src) + (size_t)(p >= 0 ? p : 0) * M::SW + blk;
+        if constexpr (M::BW == 2) {
+          const uint2 v = p >= 0 ? *reinterpret_cast<const uint2*>(row) : make_uint2(0u, 0u);
+          m[0][i] = v.x;
+          m[1][i] = v.y;
+        } else {
+          m[0][i] = p >= 0 ? *row : 0u;
+        }
       }
+#pragma unroll
+      for (int h = 0; h < M::BW; ++h) transpose32(m[h]);
+    }
+    if (M::STAGED) __syncthreads();
+    if (on) {
+#pragma unroll
+      for (int h = 0; h < M::BW; ++h)
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const int n = 32 * (blk + h) + i;
+          if (M::N % (32 * M::BW) == 0 || n < M::N) sp[n * W + word] = m[h][i];
+        }
     }
   }
 }
 
+// a + b + c = (the new a) + 2 (the result), bitwise.
+__device__ __forceinline__ uint32_t add3(uint32_t& a, uint32_t b, uint32_t c) {
+  const uint32_t carry = majority(a, b, c);
+  a = a ^ b ^ c;
+  return carry;
+}
+
 // Unsatisfied forward bonds of every replica of the tile, counted per thread in
-// CB bit planes and then added per replica into ecnt (slot i at index i).
+// CB bit planes and then added per replica into ecnt (slot i at index i).  Two sites
+// enter the planes together by full adders, so that the carries run through the upper
+// planes once per pair: 14 operations per site and word where a carry chain per site
+// takes 22.  The planes of four replicas are then read a byte each at a time (CB <= 8).
 template <int L, int W, int NP, int CB>
 __device__ __forceinline__ void count_levels_bits(const uint32_t* sp, const SiteRec* recs, int* ecnt, int word,
                                                   int part) {
   constexpr int ROWS = L * L;
-  uint32_t c[CB];
+  uint32_t c[CB > 3 ? CB : 4];
 #pragma unroll
-  for (int i = 0; i < CB; ++i) c[i] = 0;
+  for (int i = 0; i < (CB > 3 ? CB : 4); ++i) c[i] = 0;
   for (int r = part; r < ROWS; r += NP) {
     const int y = r % L, z = r / L;
     const int yp = y == L - 1 ? 0 : y + 1, zp = z == L - 1 ? 0 : z + 1;
@@ -388,61 +463,134 @@ __device__ __forceinline__ void count_levels_bits(const uint32_t* sp, const Site
     const uint32_t* pzp = sp + (size_t)(y + L * zp) * L * W + word;
     const SiteRec* rr = recs + r * L;
 #pragma unroll
-    for (int x = 0; x < L; ++x) {
-      const int xp = x == L - 1 ? 0 : x + 1;
-      const uint32_t s0 = p0[x * W];
-      const uint32_t e0 = s0 ^ p0[xp * W] ^ rr[x].jxp, e1 = s0 ^ pyp[x * W] ^ rr[x].jyp,
-                     e2 = s0 ^ pzp[x * W] ^ rr[x].jzp;
-      const uint32_t sum = e0 ^ e1 ^ e2, two = majority(e0, e1, e2);  // e0 + e1 + e2 = sum + 2 two
-      uint32_t carry = c[0] & sum;
-      c[0] ^= sum;
-      const uint32_t c1 = c[1] ^ two ^ carry;
-      carry = majority(c[1], two, carry);
-      c[1] = c1;
+    for (int x = 0; x < L; x += 2) {
+      uint32_t one[2], two[2];  // the three bonds of a site: one + 2 two
 #pragma unroll
-      for (int i = 2; i < CB; ++i) {
+      for (int h = 0; h < 2; ++h) {
+        const int xx = x + h, xp = xx == L - 1 ? 0 : xx + 1;
+        const uint32_t s0 = p0[xx * W];
+        one[h] = s0 ^ p0[xp * W] ^ rr[xx].jxp;
+        two[h] = add3(one[h], s0 ^ pyp[xx * W] ^ rr[xx].jyp, s0 ^ pzp[xx * W] ^ rr[xx].jzp);
+      }
+      const uint32_t t0 = add3(c[0], one[0], one[1]);
+      const uint32_t f0 = add3(c[1], two[0], two[1]);
+      const uint32_t f1 = c[1] & t0;
+      c[1] ^= t0;
+      uint32_t carry = add3(c[2], f0, f1);
+#pragma unroll
+      for (int i = 3; i < CB; ++i) {
         const uint32_t ci = c[i] ^ carry;
         carry &= c[i];
         c[i] = ci;
       }
     }
   }
+  if constexpr (CB <= 8) {
 #pragma unroll 1
-  for (int bb = 0; bb < 32; ++bb) {
-    const int b = (bb + word) & 31;  // lanes of a warp hit different banks
-    int k = 0;
+    for (int mm = 0; mm < 8; ++mm) {
+      const int m = (mm + word) & 7;  // replicas m, m + 8, m + 16, m + 24
+      uint32_t k4 = 0;
 #pragma unroll
-    for (int i = 0; i < CB; ++i) k |= (int)((c[i] >> b) & 1u) << i;
-    if (k) atomicAdd(&ecnt[32 * word + b], k);
+      for (int i = 0; i < CB; ++i) k4 |= ((c[i] >> m) & 0x01010101u) << i;
+#pragma unroll
+      for (int bb = 0; bb < 4; ++bb) {
+        const int b = (bb + (word >> 3)) & 3;  // lanes of a warp hit different banks
+        atomicAdd(&ecnt[32 * word + m + 8 * b], (int)((k4 >> (8 * b)) & 0xffu));
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int bb = 0; bb < 32; ++bb) {
+      const int b = (bb + word) & 31;
+      int k = 0;
+#pragma unroll
+      for (int i = 0; i < CB; ++i) k |= (int)((c[i] >> b) & 1u) << i;
+      if (k) atomicAdd(&ecnt[32 * word + b], k);
+    }
   }
 }
 
-// Write the tile back to the rows of its slots, the gather's split reversed.
-template <int L, int W, int NT, int MB>
-__device__ __forceinline__ void store_bits(const SweepArgs& a, const uint32_t* sp, int tile0) {
-  using M = RowMove<L, W, NT, MB>;
-  uint32_t* dst = a.pop.spins[1 - a.cur];
-  for (int u = threadIdx.x; u < M::STORE_UNITS; u += NT) {
-    const int word = u % W, blk = u / W * M::BW;
-    uint32_t m[M::BW][32];
-#pragma unroll
-    for (int h = 0; h < M::BW; ++h) {
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const int n = 32 * (blk + h) + i;
-        m[h][i] = n < M::N ? sp[n * W + word] : 0u;
-      }
-      transpose32(m[h]);
-    }
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      uint32_t* row = dst + (size_t)(tile0 + 32 * word + i) * M::SW + blk;
-      if constexpr (M::BW == 2)
-        *reinterpret_cast<uint2*>(row) = make_uint2(m[0][i], m[1][i]);
-      else
-        *row = m[0][i];
+// Levels of the tile's slots (ecnt), and their histogram added to the step's: the tile
+// is counted in shared memory first (hist, LEVELS words), lanes of a warp with the same
+// level by one addition, so that the step's histogram gets one global addition per
+// tile and occupied level.  With one per slot the tiles of a wave queued up at the few
+// levels a population occupies: 2.5 to 23 us per tile at L = 10, and at L = 4, beta = 3
+// (a handful of levels) 0.68 of a step's 0.73 ms at R = 1e6.
+template <int TJ, int NT, int LEVELS>
+__device__ __forceinline__ void publish_levels(const SweepArgs& a, const int* ecnt, int* hist, int tile0, int R_new) {
+  const int tid = threadIdx.x;
+  for (int k = tid; k < LEVELS; k += NT) hist[k] = 0;
+  __syncthreads();
+  const unsigned mask = warp_lanes(tid, NT);
+  for (int base = 0; base < TJ; base += NT) {  // the same iterations in every lane of a warp
+    const int i = base + tid, j = tile0 + i;
+    const bool on = i < TJ && j < R_new;
+    const int k = on ? ecnt[i] : -1;
+    const unsigned peers = __match_any_sync(mask, k);
+    if (on) {
+      a.pop.levels[j] = k;
+      if ((tid & 31) == __ffs(peers) - 1) atomicAdd(&hist[k], __popc(peers));
     }
   }
+  __syncthreads();
+  uint32_t* out = a.pop.hist + (size_t)a.t * a.n_levels;
+  for (int k = tid; k < LEVELS; k += NT)
+    if (hist[k]) atomicAdd(&out[k], (uint32_t)hist[k]);
+}
+
+// Write the tile back to the rows of its slots, the gather's split reversed.  STAGED:
+// thread 0 has issued the bulk copy of the rows [0, ROW_WORDS) of shared memory when
+// this returns (store_done waits for it); the caller synchronises either way.
+template <int L, int W, int NT, int MB>
+__device__ __forceinline__ void store_bits(const SweepArgs& a, uint32_t* sp, int tile0) {
+  using M = RowMove<L, W, NT, MB>;
+  uint32_t* dst = a.pop.spins[1 - a.cur] + (size_t)tile0 * M::SW;
+  for (int u0 = 0; u0 < M::STORE_UNITS; u0 += NT) {  // one pass when STAGED
+    const int u = u0 + threadIdx.x;
+    const bool on = u < M::STORE_UNITS;
+    uint32_t m[M::BW][32];
+    int word = 0, blk = 0;
+    if (on) {
+      move_unit<M, W, M::STORE_UNITS>(u, word, blk);
+#pragma unroll
+      for (int h = 0; h < M::BW; ++h) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const int n = 32 * (blk + h) + i;
+          m[h][i] = n < M::N ? sp[n * W + word] : 0u;
+        }
+        transpose32(m[h]);
+      }
+    }
+    if (M::STAGED) __syncthreads();
+    if (on) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        uint32_t* row = (M::STAGED ? sp : dst) + (size_t)(32 * word + i) * M::SW + blk;
+        if constexpr (M::BW == 2)
+          *reinterpret_cast<uint2*>(row) = make_uint2(m[0][i], m[1][i]);
+        else
+          *row = m[0][i];
+      }
+    }
+  }
+  if constexpr (M::STAGED) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the rows before the copy reads them
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
+                   "r"((uint32_t)__cvta_generic_to_shared(sp)), "r"(4 * M::ROW_WORDS)
+                   : "memory");
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      if (!M::POST_BEHIND) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    }
+  }
+}
+
+// The bulk copy of store_bits is complete (the thread that issued it waits).
+template <typename M>
+__device__ __forceinline__ void store_done() {
+  if (M::STAGED && threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 // Families (a7) of the tile's new slots, so that a step needs no family launch
@@ -528,11 +676,12 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int
   int* rowtab = slots + S::SLOTS;  // [NP][RPP][8]: word offsets of a row and its four neighbour rows, its first site
   const int tid = threadIdx.x, word = tid % W, part = tid / W;
   Deferred* dq = queues + (S::DEFER ? (tid >> 5) * kQueueCap : 0);
-  init_tables<L>(a, recs, tid, NT);
+  using M = RowMove<L, W, NT, MB>;
   if constexpr (S::DEFER) fill_row_table<L, W, NP>(rowtab, tid, NT);
   for (int i = tid; i < TJ; i += NT) slots[33 * (i >> 5) + (i & 31)] = parent_of(a, tile0 + i, R_new);
   __syncthreads();
   gather_bits<L, W, NT, MB>(a, sp, slots);
+  init_tables<L>(a, recs, tid, NT);
   __syncthreads();
   for (int i = tid; i < S::SLOTS; i += NT) slots[i] = 0;
   __syncthreads();
@@ -575,11 +724,15 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int
   }
   count_levels_bits<L, W, NP, S::CB>(sp, recs, slots, word, part);
   __syncthreads();
-  publish_levels<TJ>(a, slots, tile0, R_new, tid, NT);
   store_bits<L, W, NT, MB>(a, sp, tile0);
-  if (!a.fam) return;
-  __syncthreads();  // every shared array is dead now: the family pass takes the space
-  tile_families<TJ, NT>(a, reinterpret_cast<int*>(sm), tile0, R_new, tid);
+  if (!M::POST_BEHIND) __syncthreads();  // the words (or their rows) are dead
+  int* post = reinterpret_cast<int*>(sm) + M::POST;
+  publish_levels<TJ, NT, M::LEVELS>(a, slots, post, tile0, R_new);
+  if (a.fam) {
+    __syncthreads();  // the level counts are dead
+    tile_families<TJ, NT>(a, post, tile0, R_new, tid);
+  }
+  store_done<M>();
 }
 
 // Bit-sliced sweep kernel (+-1 couplings): one tile per CTA.
