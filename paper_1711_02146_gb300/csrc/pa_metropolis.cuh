@@ -75,6 +75,15 @@ __device__ __forceinline__ void mulhilo(uint32_t m, uint32_t a, uint32_t& hi, ui
   lo = (uint32_t)p;
 }
 
+// The site/step part of Philox rounds 1-3: ua and ub of a SiteRec.
+__device__ __forceinline__ uint2 site_philox(uint32_t n, uint32_t t, const MetropolisArgs& a) {
+  uint32_t hi0, lo0, hi1, lo1;
+  mulhilo(kM0, n >> 1, hi0, lo0);
+  const uint32_t c1 = hi0 ^ t ^ a.k1[0];
+  mulhilo(kM1, c1, hi1, lo1);
+  return make_uint2(hi1 ^ a.k0[1], lo1 ^ a.k0[2]);
+}
+
 // The record of site n at step t; jtab: the forward-bond masks (non-zero for J = -1).
 __device__ __forceinline__ SiteRec site_record(int L, int n, const uint32_t* __restrict__ jtab, uint32_t t,
                                                const MetropolisArgs& a) {
@@ -89,12 +98,9 @@ __device__ __forceinline__ SiteRec site_record(int L, int n, const uint32_t* __r
   r.jxm = jtab[4 * nxm + 0] ? ~0u : 0u;
   r.jym = jtab[4 * nym + 1] ? ~0u : 0u;
   r.jzm = jtab[4 * nzm + 2] ? ~0u : 0u;
-  uint32_t hi0, lo0, hi1, lo1;
-  mulhilo(kM0, (uint32_t)n >> 1, hi0, lo0);
-  const uint32_t c1 = hi0 ^ t ^ a.k1[0];
-  mulhilo(kM1, c1, hi1, lo1);
-  r.ua = hi1 ^ a.k0[1];
-  r.ub = lo1 ^ a.k0[2];
+  const uint2 u = site_philox((uint32_t)n, t, a);
+  r.ua = u.x;
+  r.ub = u.y;
   return r;
 }
 
@@ -123,12 +129,12 @@ __device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c)
 
 // One Philox block (rounds 3..10 from the hoisted parts) of site h, uc = lo(M0 h),
 // for the thread's group of block index b (its ThreadPhilox tp).
-__device__ __forceinline__ void philox_block(uint32_t uc, const SiteRec& sr, const ThreadPhilox& tp, const uint32_t* k0,
-                                             const uint32_t* k1, uint32_t (&w)[4]) {
+__device__ __forceinline__ void philox_block(uint32_t uc, uint32_t ua, uint32_t ub, const ThreadPhilox& tp,
+                                             const uint32_t* k0, const uint32_t* k1, uint32_t (&w)[4]) {
   uint32_t hh, l, h2, l2;
   mulhilo(kM1, tp.tb ^ uc, hh, l);
-  mulhilo(kM0, sr.ua ^ tp.ta, h2, l2);
-  w[0] = hh ^ sr.ub;
+  mulhilo(kM0, ua ^ tp.ta, h2, l2);
+  w[0] = hh ^ ub;
   w[1] = l;
   w[2] = h2 ^ tp.tdk;
   w[3] = l2;
@@ -143,6 +149,11 @@ __device__ __forceinline__ void philox_block(uint32_t uc, const SiteRec& sr, con
     w[2] = n2;
     w[3] = l2;
   }
+}
+
+__device__ __forceinline__ void philox_block(uint32_t uc, const SiteRec& sr, const ThreadPhilox& tp, const uint32_t* k0,
+                                             const uint32_t* k1, uint32_t (&w)[4]) {
+  philox_block(uc, sr.ua, sr.ub, tp, k0, k1, w);
 }
 
 // The plane's threshold bit of each replica of a word (SweepArgs::tm), from bits

@@ -133,6 +133,7 @@ constexpr int kQueueCap = 64;  // words a warp queues; it finishes 32 of them as
 
 template <int L, int W, int NT, int MB>
 struct BitShape {
+  static constexpr int LL = L, WW = W, THREADS = NT, CTAS = MB;
   static constexpr int N = L * L * L;
   static constexpr int ROWS = L * L;
   static constexpr int NP = NT / W;       // row partitions
@@ -151,6 +152,7 @@ struct BitShape {
                                 (size_t)MB * (SMEM_TILE + SMEM_QUEUES + SMEM_ROWS + 1024) <= 233472;
   static constexpr int NQ = DEFER ? NT / 32 : 0;  // one queue per warp
   static constexpr size_t SMEM = SMEM_TILE + (DEFER ? SMEM_QUEUES + SMEM_ROWS : 0);
+  static constexpr size_t SLOT_TABLE = SMEM_TILE - (size_t)SLOTS * 4 + (DEFER ? SMEM_QUEUES : 0);  // its offset
   static_assert(NT % W == 0 && 32 % W == 0 && NT <= 1024, "threads must tile the words of a row");
   static_assert(L % 2 == 0 && L / 2 <= 8, "even L up to 16");
   static_assert(NP % 2 == 0 && (ROWS / 2) % (NP / 2) == 0, "row partitions must split each parity class");
@@ -342,34 +344,34 @@ __device__ __forceinline__ void sweep_rows_bits_dq(uint32_t* sp, int word, const
 // one bulk copy of contiguous memory.  Otherwise each thread reads and writes its
 // pieces of 4 BW bytes in global memory.  At L = 10 (1024 slots, 128 KB) the pieces
 // took 10.5 us to gather and 11 to 21 us to store.
-template <int L, int W, int NT, int MB>
-struct RowMove : Row<L> {
-  using S = BitShape<L, W, NT, MB>;
-  using Row<L>::N;
-  using Row<L>::SW;
-  using Row<L>::NB;
+// S: the tile's shape (lattice size LL, WW words per site, THREADS, CTAS per SM, and the
+// bytes from the tile's words to its slot table).
+template <typename S>
+struct RowMove : Row<S::LL> {
+  using Row<S::LL>::N;
+  using Row<S::LL>::SW;
+  using Row<S::LL>::NB;
+  static constexpr int W = S::WW, NT = S::THREADS, MB = S::CTAS;
   static constexpr int BW = SW % 2 == 0 && NT * MB <= 640 ? 2 : 1;
   static constexpr int GATHER_UNITS = W * ((NB + BW - 1) / BW);
   static constexpr int STORE_UNITS = W * (SW / BW);  // the padding of a row too: its bits stay 0
-  static constexpr size_t SLOT_TABLE = (size_t)N * W * 4 + (size_t)N * sizeof(SiteRec) +
-                                       (size_t)S::NQ * kQueueCap * sizeof(Deferred);  // its offset in bytes
   static constexpr int ROW_WORDS = 32 * W * SW;
-  static constexpr bool STAGED = STORE_UNITS <= NT && (size_t)ROW_WORDS * 4 <= SLOT_TABLE;
+  static constexpr bool STAGED = STORE_UNITS <= NT && (size_t)ROW_WORDS * 4 <= S::SLOT_TABLE;
   // Shared memory of the measurements after the store (level counts of the tile, then
   // the families): behind the rows while they are copied out, or in their place.
   static constexpr int LEVELS = 3 * N + 1;
   static constexpr int FAM_WORDS = ((32 * W + 1 + W + 2) & ~1) + 128;
   static constexpr int POST_WORDS = LEVELS > FAM_WORDS ? LEVELS : FAM_WORDS;
-  static constexpr bool POST_BEHIND = STAGED && (size_t)(ROW_WORDS + POST_WORDS) * 4 <= SLOT_TABLE;
+  static constexpr bool POST_BEHIND = STAGED && (size_t)(ROW_WORDS + POST_WORDS) * 4 <= S::SLOT_TABLE;
   static constexpr int POST = POST_BEHIND ? ROW_WORDS : 0;
 };
 
 // The unit's word column and first row word.  Neighbouring lanes take neighbouring
 // word columns, and (STAGED) row words one step apart, which spreads both the rows and
 // the words over the banks.
-template <typename M, int W, int UNITS>
+template <typename M, int UNITS>
 __device__ __forceinline__ void move_unit(int u, int& word, int& blk) {
-  constexpr int NBLK = UNITS / W;
+  constexpr int W = M::W, NBLK = UNITS / W;
   word = u % W;
   blk = (M::STAGED ? (u / W + word) % NBLK : u / W) * M::BW;
 }
@@ -385,9 +387,10 @@ __device__ __forceinline__ void copy_async(uint32_t dst, const void* src, bool z
 // holds the tile's parents (-1 past R~), slot i at index 33 (i >> 5) + (i & 31).
 // Ends with the words written but not yet synchronised; the site records may be
 // written from then on, not before (STAGED).
-template <int L, int W, int NT, int MB>
+template <typename S>
 __device__ __forceinline__ void gather_bits(const SweepArgs& a, uint32_t* sp, const int* spar) {
-  using M = RowMove<L, W, NT, MB>;
+  using M = RowMove<S>;
+  constexpr int W = M::W, NT = M::NT;
   const uint32_t* src = a.pop.spins[a.cur];
   if constexpr (M::STAGED) {
     constexpr int CW = M::SW % 4 == 0 ? 4 : M::SW;  // words per copy
@@ -407,7 +410,7 @@ __device__ __forceinline__ void gather_bits(const SweepArgs& a, uint32_t* sp, co
     uint32_t m[M::BW][32];
     int word = 0, blk = 0;
     if (on) {
-      move_unit<M, W, M::GATHER_UNITS>(u, word, blk);
+      move_unit<M, M::GATHER_UNITS>(u, word, blk);
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
         const int p = M::STAGED ? 32 * word + i : spar[33 * word + i];
@@ -541,9 +544,10 @@ __device__ __forceinline__ void publish_levels(const SweepArgs& a, const int* ec
 // Write the tile back to the rows of its slots, the gather's split reversed.  STAGED:
 // thread 0 has issued the bulk copy of the rows [0, ROW_WORDS) of shared memory when
 // this returns (store_done waits for it); the caller synchronises either way.
-template <int L, int W, int NT, int MB>
+template <typename S>
 __device__ __forceinline__ void store_bits(const SweepArgs& a, uint32_t* sp, int tile0) {
-  using M = RowMove<L, W, NT, MB>;
+  using M = RowMove<S>;
+  constexpr int W = M::W, NT = M::NT;
   uint32_t* dst = a.pop.spins[1 - a.cur] + (size_t)tile0 * M::SW;
   for (int u0 = 0; u0 < M::STORE_UNITS; u0 += NT) {  // one pass when STAGED
     const int u = u0 + threadIdx.x;
@@ -551,7 +555,7 @@ __device__ __forceinline__ void store_bits(const SweepArgs& a, uint32_t* sp, int
     uint32_t m[M::BW][32];
     int word = 0, blk = 0;
     if (on) {
-      move_unit<M, W, M::STORE_UNITS>(u, word, blk);
+      move_unit<M, M::STORE_UNITS>(u, word, blk);
 #pragma unroll
       for (int h = 0; h < M::BW; ++h) {
 #pragma unroll
@@ -676,11 +680,11 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int
   int* rowtab = slots + S::SLOTS;  // [NP][RPP][8]: word offsets of a row and its four neighbour rows, its first site
   const int tid = threadIdx.x, word = tid % W, part = tid / W;
   Deferred* dq = queues + (S::DEFER ? (tid >> 5) * kQueueCap : 0);
-  using M = RowMove<L, W, NT, MB>;
+  using M = RowMove<S>;
   if constexpr (S::DEFER) fill_row_table<L, W, NP>(rowtab, tid, NT);
   for (int i = tid; i < TJ; i += NT) slots[33 * (i >> 5) + (i & 31)] = parent_of(a, tile0 + i, R_new);
   __syncthreads();
-  gather_bits<L, W, NT, MB>(a, sp, slots);
+  gather_bits<S>(a, sp, slots);
   init_tables<L>(a, recs, tid, NT);
   __syncthreads();
   for (int i = tid; i < S::SLOTS; i += NT) slots[i] = 0;
@@ -724,7 +728,7 @@ __device__ __forceinline__ void sweep_tile(const SweepArgs& a, uint32_t* sm, int
   }
   count_levels_bits<L, W, NP, S::CB>(sp, recs, slots, word, part);
   __syncthreads();
-  store_bits<L, W, NT, MB>(a, sp, tile0);
+  store_bits<S>(a, sp, tile0);
   if (!M::POST_BEHIND) __syncthreads();  // the words (or their rows) are dead
   int* post = reinterpret_cast<int*>(sm) + M::POST;
   publish_levels<TJ, NT, M::LEVELS>(a, slots, post, tile0, R_new);
