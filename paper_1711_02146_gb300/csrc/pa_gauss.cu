@@ -274,19 +274,37 @@ __global__ void k_g_tables(const double* __restrict__ dbeta_dev, double dbeta_va
   T[m] = g_table_entry(dbeta_dev ? *dbeta_dev : dbeta_val, m);
 }
 
-// The whole bisection in one cooperative launch (every block resident, blocks of
-// kBisectThreads): each halving is one pass over the old population for the
-// weights of mid and their chunk partial sums, a grid barrier whose last block to
-// arrive adds the partial sums (block_total, the order of tree_total) into S', a
-// pass for the culling terms (S' - R w_i)_+ and their chunk partial sums, and a
-// second such barrier for their total; every block then takes the same decision.
-// The weight tables of the two possible next midpoints are built during the second
-// pass, into the two table sets not in use, T2 only up to the entry of the largest
-// d = E_i - E_min (found once, before the first halving).  The values, sums and
-// decisions are those of the launch-per-trial path (k_g_tables, k_g_weights,
-// k_g_tau), so both give the same lo, hi and mid.
-constexpr int kBisectThreads = 256;
+// The whole bisection in one cooperative launch (every block resident, one per SM).
+// The values, sums and decisions are those of the launch-per-trial path (k_g_tables,
+// k_g_weights, k_g_tau): a trial is one pass over the old population for the weights of
+// the trial's dbeta and their chunk sums, a grid barrier whose last block to arrive adds
+// the chunk sums (block_total, the order of tree_total) into S', a pass for the culling
+// terms (S' - R w_i)_+ and their chunk sums, and a second such barrier for their total;
+// every block then takes the same decision.  Each warp keeps the energies and weights of
+// its first kBisectKeep chunks in registers, and a block the trial's weight tables in
+// shared memory, copied from global memory where all blocks have built them together
+// (T2 only up to the entry of the largest d = E_i - E_min): three scattered 8-byte reads
+// per replica and trial went to L2 before.
+//
+// Most halvings need no trial.  The culling fraction e is the mean of (1 - tau_i)_+, with
+// p_i = tau_i / R the Boltzmann weights of the move normalised over the R~ replicas, and
+// e rises with dbeta from dbeta0 on if the relative entropy K(dbeta0) of (p_i) to the
+// uniform law exceeds ln(R~/R): a replica that is culled then has an energy above the
+// mean under (p_i), so every term of e rises, and dK/d dbeta = dbeta Var(E) >= 0 keeps
+// the condition.  By Pinsker's inequality K >= 2 v^2, and the total variation v is e up
+// to x = |R~/R - 1|, so e(dbeta0) - x >= 0.8 sqrt(x) suffices (monotone_from).  A few
+// secant steps from the slope of a normal law (Eq. eps: e = dbeta sigma / sqrt(2 pi))
+// therefore find a point below which every midpoint from dbeta0 on is accepted and one
+// above which every midpoint is rejected, each by more than the rounding of e (about
+// 1e-14; kTrialMargin), and only the midpoints between them (and below dbeta0) are tried.
+// That leaves some 25 of 58 trials; a trial takes about 20 us instead of 55 at R = 1e6
+// (FP64 pipe: 7 operations per replica, 10 us).
+constexpr int kBisectThreads = 512;
 constexpr int kBisectWarps = kBisectThreads / 32;
+constexpr int kBisectKeep = 2;
+constexpr int kBisectSecant = 8;                    // secant trials at most
+constexpr double kTrialMargin = 2e-13;
+constexpr size_t kBisectSmem = sizeof(double) * (size_t)kGTableWeights;
 constexpr int kBisectMaxChunks = kChunk * kChunk;  // block_total keeps two tree levels
 constexpr unsigned kBarrierSpins = 1u << 22;       // polls of one barrier wait (about 0.5 s at most)
 // words of the barrier block: arrivals, generation, error, largest d, S', culling sum
@@ -369,21 +387,57 @@ __device__ __forceinline__ double bar_double(const unsigned long long* bar, int 
 
 struct BisectArgs {
   PopDev P;                 // population 0 decides the step
-  double* b;                // {lo, hi, mid, state}: in, and out (state 1 done, -1 a barrier wait ran out)
+  double* b;                // {lo, hi, mid, state}, out: state 1 done, 2 the whole range is accepted, -1 a wait ran out
   double* T;                // three sets of kGTableWeights table entries
   double* part1;            // [n_chunks] chunk partial sums of the culling terms (those of the weights in P.part)
   unsigned long long* bar;  // kBarWords words, zero at launch
   unsigned spins;           // polls of a barrier wait
   int withheld;             // block that does not arrive at the first barrier (-1: none; tests)
   int t, R, halvings;
+  double range;             // the remaining dbeta
   double target;
 };
 
-__global__ void __launch_bounds__(kBisectThreads, 4) k_g_bisect(BisectArgs a) {
+// The bisection's interval, next midpoint and halvings done.
+struct Halving {
+  double lo, hi, mid;
+  int h;
+  bool done;
+  __device__ __forceinline__ void decide(bool accept) {
+    if (accept)
+      lo = mid;
+    else
+      hi = mid;
+    mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
+    ++h;
+    // the fixed point of k_g_tau: every later halving evaluates a point already decided
+    if (mid == hi || (mid == lo && lo > 0.0)) done = true;
+  }
+};
+
+// What the trials so far say of other points: accepted in [from, below], rejected from
+// max(from, above) on.
+struct Known {
+  double from, below, above;
+  __device__ __forceinline__ void trial(double x, double e, double target, double excess) {
+    if (e - excess >= 0.8 * sqrt(excess) && x < from) from = x;  // monotone_from
+    if (e <= target - kTrialMargin && x > below) below = x;
+    if (e >= target + kTrialMargin && x < above) above = x;
+  }
+  // Halvings whose midpoint is decided already.
+  __device__ __forceinline__ void settle(Halving& s, int halvings) const {
+    while (!s.done && s.h < halvings && s.mid >= from && (s.mid <= below || s.mid >= above)) s.decide(s.mid <= below);
+    if (s.h >= halvings) s.done = true;
+  }
+};
+
+__global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
+  extern __shared__ double tab[];  // the current trial's tables
   __shared__ double lvl[kChunk];
   const PopDev& P = a.P;
   const int R_old = P.rec[a.t - 1].R_tilde;
-  const long long Emin = P.grec[a.t - 1].E_min;
+  const GRec& old = P.grec[a.t - 1];
+  const long long Emin = old.E_min;
   const int nch = (R_old + kChunk - 1) / kChunk;
   const int lane = threadIdx.x & 31;
   const int gwarp = blockIdx.x * kBisectWarps + (threadIdx.x >> 5);
@@ -391,7 +445,19 @@ __global__ void __launch_bounds__(kBisectThreads, 4) k_g_bisect(BisectArgs a) {
   const int gtid = blockIdx.x * kBisectThreads + threadIdx.x;
   const int n_threads = gridDim.x * kBisectThreads;
   const double R = (double)a.R;
-  double lo = a.b[0], hi = a.b[1], mid = a.b[2];
+  // the warp's first chunks: d = E - E_min as its low 24 bits and the rest (-1: no replica)
+  uint32_t dl[kBisectKeep][8];
+  int dh[kBisectKeep][8];
+  double w[kBisectKeep][8];
+#pragma unroll
+  for (int j = 0; j < kBisectKeep; ++j)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const long long i = (long long)(gwarp + j * n_warps) * kChunk + lane + 32 * k;
+      const long long d = i < R_old ? P.E64[i] - Emin : -1;
+      dl[j][k] = (uint32_t)d & 0xFFFFFFu;
+      dh[j][k] = i < R_old ? (int)(d >> 24) : -1;
+    }
   unsigned long long dmax = 0;  // the largest d: T2 beyond its entry is never read
   for (int i = gtid; i < R_old; i += n_threads) {
     const unsigned long long d = (unsigned long long)(P.E64[i] - Emin);
@@ -404,12 +470,32 @@ __global__ void __launch_bounds__(kBisectThreads, 4) k_g_bisect(BisectArgs a) {
   if (lane == 0 && dmax) atomicMax(&a.bar[kBarDmax], dmax);
   bool ok = grid_barrier(a.bar, a.spins, (int)blockIdx.x == a.withheld);
   const int n_tab = 8192 + (int)min(8191ull, ((volatile unsigned long long*)a.bar)[kBarDmax] >> 24) + 1;
-  for (int m = gtid; m < n_tab; m += n_threads) a.T[m] = g_table_entry(mid, m);
-  int cur = 0;
-  ok = ok && grid_barrier(a.bar, a.spins);
-  for (int h = 0; h < a.halvings && ok; ++h) {
-    const double* Tc = a.T + (size_t)cur * kGTableWeights;
-    for (int c = gwarp; c < nch; c += n_warps) {  // weights of mid and their chunk sums
+
+  auto build = [&](int set, double db) {  // this block's share of the tables of db
+    for (int m = gtid; m < n_tab; m += n_threads) __stcg(a.T + (size_t)set * kGTableWeights + m, g_table_entry(db, m));
+  };
+  auto weight = [&](uint32_t lo, int hi) {
+    return __dmul_rn(__dmul_rn(tab[8192 + hi], tab[4096 + (lo >> 12)]), tab[lo & 4095u]);
+  };
+  // The culling fraction of the dbeta whose tables are in `set` (built and behind a
+  // barrier); `between` runs while the sums of the weights are known.
+  auto trial = [&](int set, auto between) -> double {
+    __syncthreads();
+    const double2* src = reinterpret_cast<const double2*>(a.T + (size_t)set * kGTableWeights);
+    for (int m = threadIdx.x; m < (n_tab + 1) / 2; m += kBisectThreads) reinterpret_cast<double2*>(tab)[m] = __ldcg(src + m);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kBisectKeep; ++j) {
+      const int c = gwarp + j * n_warps;
+      if (c < nch) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = w[j][k] = dh[j][k] >= 0 ? weight(dl[j][k], dh[j][k]) : 0.0;
+        const double sum = group8(v);
+        if (lane == 0) __stcg(P.part + c, sum);
+      }
+    }
+    for (int c = gwarp + kBisectKeep * n_warps; c < nch; c += n_warps) {
       double v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
@@ -417,58 +503,141 @@ __global__ void __launch_bounds__(kBisectThreads, 4) k_g_bisect(BisectArgs a) {
         v[k] = 0.0;
         if (i < R_old) {
           const long long d = P.E64[i] - Emin;
-          v[k] = __dmul_rn(__dmul_rn(__ldcg(Tc + 8192 + (d >> 24)), __ldcg(Tc + 4096 + ((d >> 12) & 4095))),
-                           __ldcg(Tc + (d & 4095)));
+          v[k] = weight((uint32_t)d & 0xFFFFFFu, (int)(d >> 24));
           __stcg(P.w + i, v[k]);
         }
       }
       const double sum = group8(v);
       if (lane == 0) __stcg(P.part + c, sum);
     }
-    if (!grid_barrier(a.bar, a.spins, false, P.part, nch, kBarS, lvl)) break;
+    if (!grid_barrier(a.bar, a.spins, false, P.part, nch, kBarS, lvl)) {
+      ok = false;
+      return 0.0;
+    }
     const double S = bar_double(a.bar, kBarS);
     const long long S_bits = __double_as_longlong(S);
-    const int s_acc = cur == 2 ? 0 : cur + 1, s_rej = cur == 0 ? 2 : cur - 1;
-    const double m_acc = __dmul_rn(0.5, __dadd_rn(mid, hi)), m_rej = __dmul_rn(0.5, __dadd_rn(lo, mid));
-    for (int m = gtid; m < 2 * n_tab; m += n_threads) {  // both possible next tables
-      const bool acc = m < n_tab;
-      const int e = acc ? m : m - n_tab;
-      a.T[(size_t)(acc ? s_acc : s_rej) * kGTableWeights + e] = g_table_entry(acc ? m_acc : m_rej, e);
+    between();
+    // rw < S' compared as the bit patterns of two non-negative doubles (an integer
+    // comparison, the same order)
+    auto culled = [&](double wi) {
+      const double rw = __dmul_rn(R, wi);
+      return __double_as_longlong(rw) < S_bits ? __dsub_rn(S, rw) : 0.0;
+    };
+#pragma unroll
+    for (int j = 0; j < kBisectKeep; ++j) {
+      const int c = gwarp + j * n_warps;
+      if (c < nch) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = dh[j][k] >= 0 ? culled(w[j][k]) : 0.0;
+        const double sum = group8(v);
+        if (lane == 0) __stcg(a.part1 + c, sum);
+      }
     }
-    for (int c = gwarp; c < nch; c += n_warps) {  // culling terms and their chunk sums
+    for (int c = gwarp + kBisectKeep * n_warps; c < nch; c += n_warps) {
       double v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         const int i = c * kChunk + lane + 32 * k;
-        v[k] = 0.0;
-        if (i < R_old) {
-          // rw < S' compared as the bit patterns of two non-negative doubles (an
-          // integer comparison, the same order)
-          const double rw = __dmul_rn(R, __ldcg(P.w + i));
-          if (__double_as_longlong(rw) < S_bits) v[k] = __dsub_rn(S, rw);
-        }
+        v[k] = i < R_old ? culled(__ldcg(P.w + i)) : 0.0;
       }
       const double sum = group8(v);
       if (lane == 0) __stcg(a.part1 + c, sum);
     }
-    if (!grid_barrier(a.bar, a.spins, false, a.part1, nch, kBarCull, lvl)) break;
-    const double e = __ddiv_rn(__ddiv_rn(bar_double(a.bar, kBarCull), S), R);
-    if (e <= a.target) {
-      lo = mid;
-      cur = s_acc;
-    } else {
-      hi = mid;
-      cur = s_rej;
+    if (!grid_barrier(a.bar, a.spins, false, a.part1, nch, kBarCull, lvl)) {
+      ok = false;
+      return 0.0;
     }
-    mid = __dmul_rn(0.5, __dadd_rn(lo, hi));
-    // the fixed point of k_g_tau: every later halving evaluates a point already decided
-    if (mid == hi || (mid == lo && lo > 0.0)) break;
+    return __ddiv_rn(__ddiv_rn(bar_double(a.bar, kBarCull), S), R);
+  };
+  auto nothing = [] {};
+  auto trial_at = [&](double x) -> double {
+    build(0, x);
+    if (!grid_barrier(a.bar, a.spins)) {
+      ok = false;
+      return 0.0;
+    }
+    return trial(0, nothing);
+  };
+
+  Halving s{0.0, a.range, __dmul_rn(0.5, a.range), 0, false};
+  double e_range = 0.0;
+  if (ok) e_range = trial_at(a.range);
+  const bool all = ok && e_range <= a.target;
+  if (ok && !all) {
+    const double excess = fabs((double)R_old / R - 1.0);
+    Known known{1.0 / 0.0, 0.0, 1.0 / 0.0};
+    known.trial(a.range, e_range, a.target, excess);
+    if (a.target - excess > 0.8 * sqrt(excess)) {
+      // secant steps on e(x) - target, kept inside the tightest bracket seen
+      const double n = (double)R_old, mean = (double)old.sum_E / n;
+      const double sq = ((double)old.sum_E2_hi * 0x1p64 + (double)old.sum_E2_lo) / n;
+      const double sigma = sqrt(fmax(sq - mean * mean, 0.0)) * 0x1p-20;
+      double xa = 0.0, xb = a.range, px = 0.0, pe = 0.0, slope = 0.0;
+      double x = a.target * 2.5066282746310002 / sigma;  // sqrt(2 pi)
+      if (!(x > 0.0 && x < 0.5 * a.range)) x = 0.5 * a.range;
+      bool near = false;
+      for (int k = 0; k < kBisectSecant && ok && !near; ++k) {
+        const double e = trial_at(x);
+        if (!ok) break;
+        known.trial(x, e, a.target, excess);
+        if (e <= a.target)
+          xa = fmax(xa, x);
+        else
+          xb = fmin(xb, x);
+        slope = (e - pe) / (x - px);  // the first step: from e(0) = 0
+        px = x;
+        pe = e;
+        near = fabs(e - a.target) < 1e-10;
+        double y = x - (e - a.target) / slope;
+        if (!(y > xa && y < xb)) y = 0.5 * (xa + xb);
+        x = y;
+      }
+      // a point on either side of the root, as near as the rounding of e allows
+      const double dx = 3.0 * kTrialMargin / slope;
+      if (ok && near && slope > 0.0 && known.below < x - dx) known.trial(x - dx, trial_at(x - dx), a.target, excess);
+      if (ok && near && slope > 0.0 && known.above > x + dx) known.trial(x + dx, trial_at(x + dx), a.target, excess);
+    }
+    known.settle(s, a.halvings);
+    int cur = 0;
+    if (ok && !s.done) {
+      build(cur, s.mid);
+      ok = grid_barrier(a.bar, a.spins);
+    }
+    while (ok && !s.done) {
+      Halving acc = s, rej = s;
+      acc.decide(true);
+      rej.decide(false);
+      known.settle(acc, a.halvings);
+      known.settle(rej, a.halvings);
+      const int s_acc = cur == 2 ? 0 : cur + 1, s_rej = cur == 0 ? 2 : cur - 1;
+      const double x = s.mid;
+      const double e = trial(cur, [&] {  // both possible next tables, while the culling terms are summed
+        if (!acc.done) build(s_acc, acc.mid);
+        if (!rej.done) build(s_rej, rej.mid);
+      });
+      if (!ok) break;
+      const bool accept = e <= a.target;
+      s = accept ? acc : rej;
+      cur = accept ? s_acc : s_rej;
+      const double from = known.from;
+      known.trial(x, e, a.target, excess);
+      // midpoints that this trial has decided: their tables come after the next undecided one's
+      if (known.from < from && !s.done) {
+        const double mid = s.mid;
+        known.settle(s, a.halvings);
+        if (!s.done && s.mid != mid) {
+          build(cur, s.mid);
+          ok = grid_barrier(a.bar, a.spins);
+        }
+      }
+    }
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    a.b[0] = lo;
-    a.b[1] = hi;
-    a.b[2] = mid;
-    a.b[3] = ((volatile unsigned long long*)a.bar)[kBarError] != 0ull ? -1.0 : 1.0;
+    a.b[0] = s.lo;
+    a.b[1] = s.hi;
+    a.b[2] = s.mid;
+    a.b[3] = !ok || ((volatile unsigned long long*)a.bar)[kBarError] != 0ull ? -1.0 : all ? 2.0 : 1.0;
   }
 }
 
@@ -711,17 +880,18 @@ int g_bisect_blocks(const RunGeom& g) {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop ||
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g_bisect, kBisectThreads, 0) != cudaSuccess) {
+      cudaFuncSetAttribute(k_g_bisect, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBisectSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_g_bisect, kBisectThreads, kBisectSmem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   const int want = blocks_for(g.n_chunks, kBisectWarps);  // one chunk per warp when the device holds them
-  return std::max(1, std::min(want, per_sm * n_sm));
+  return std::min(want, per_sm * n_sm);
 }
 
 int launch_g_bisect_fused(const RunGeom& g, PopDev* pops, int t, double* tables, double* part1,
-                          unsigned long long* bar, double* b, double target, int halvings, int n_blocks,
-                          int withheld, void* stream) {
+                          unsigned long long* bar, double* b, double range, double target, int halvings,
+                          int n_blocks, int withheld, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   BisectArgs a;
   a.P = pops[0];
@@ -732,13 +902,15 @@ int launch_g_bisect_fused(const RunGeom& g, PopDev* pops, int t, double* tables,
   a.t = t;
   a.R = g.R;
   a.halvings = halvings;
+  a.range = range;
   a.target = target;
   a.withheld = withheld;
   a.spins = withheld >= 0 ? 4096u : kBarrierSpins;
   cudaError_t e = cudaMemsetAsync(bar, 0, kBarWords * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return (int)e;
   void* args[] = {&a};
-  e = cudaLaunchCooperativeKernel((const void*)k_g_bisect, dim3((unsigned)n_blocks), dim3(kBisectThreads), args, 0, s);
+  e = cudaLaunchCooperativeKernel((const void*)k_g_bisect, dim3((unsigned)n_blocks), dim3(kBisectThreads), args,
+                                  kBisectSmem, s);
   return (int)e;
 }
 

@@ -211,16 +211,18 @@ int launch_g_tables(const double* dbeta_dev, double dbeta_val, double* T, void* 
 // (mid equal to a point already decided), after which the halvings do no work.
 int launch_g_bisect(const RunGeom& g, PopDev* pops, int t, double* T, double* b, double target, int halvings,
                     void* stream);
-// The same halvings in one cooperative launch of n_blocks blocks (g_bisect_blocks:
-// 0 when the device or the population size does not allow it): tables = three sets
-// of kGTableWeights entries, part1 = n_chunks partial sums, bar = 8 words (barrier
-// and totals, cleared on the stream first).  On return b = {lo, hi, mid, state}, state -1 when
-// a grid barrier wait ran out (the interval is then not to be used).  withheld >= 0 (tests):
-// that block does not arrive at the first barrier and the waits poll 4096 times, so they run out.
+// The trial of the whole range and, where it is not accepted, the same halvings from
+// {0, range} in one cooperative launch of n_blocks blocks (g_bisect_blocks: 0 when the
+// device or the population size does not allow it): tables = three sets of
+// kGTableWeights entries, part1 = n_chunks partial sums, bar = 8 words (barrier and
+// totals, cleared on the stream first).  On return b = {lo, hi, mid, state}, state 2 when
+// the range is accepted, -1 when a grid barrier wait ran out (the interval is then not
+// to be used).  withheld >= 0 (tests): that block does not arrive at the first barrier
+// and the waits poll 4096 times, so they run out.
 int g_bisect_blocks(const RunGeom& g);
 int launch_g_bisect_fused(const RunGeom& g, PopDev* pops, int t, double* tables, double* part1,
-                          unsigned long long* bar, double* b, double target, int halvings, int n_blocks,
-                          int withheld, void* stream);
+                          unsigned long long* bar, double* b, double range, double target, int halvings,
+                          int n_blocks, int withheld, void* stream);
 int launch_overlap(const RunGeom& g, PopDev* pops, int cur, int t, unsigned long long* qhist, void* stream);
 int overlap_blocks(const RunGeom& g);  // blocks of the overlap of one pair of populations
 

@@ -657,28 +657,36 @@ int choose_dbeta_gauss(pa_ctx* c, double* dbeta) {
   const double rem = c->cfg.beta_max - c->betas[(size_t)c->t];
   const double target = c->cfg.eps_target;
   double b[4] = {0.0, rem, rem, 0.0};
-  int rc = copy_h2d(c, c->gbis, b, sizeof b);
-  if (rc == PA_OK) rc = launch_rc(pa::launch_g_tables(c->gbis + 2, 0.0, c->gw, c->stream));
-  if (rc == PA_OK) rc = launch_rc(pa::launch_g_eps_trial(c->g, c->pops, t, c->gw, c->stream));
-  double e = 0.0;
-  if (rc == PA_OK) rc = copy_d2h(c, &e, &c->pops[0].rec[t].eps_expected, sizeof(double));
-  if (rc != PA_OK) return rc;
-  if (e <= target) {
-    *dbeta = rem;
-    return PA_OK;
-  }
-  b[2] = 0.5 * (b[0] + b[1]);
-  rc = copy_h2d(c, c->gbis, b, sizeof b);
   if (c->gbis_blocks < 0) c->gbis_blocks = pa::g_bisect_blocks(c->g);
-  if (rc == PA_OK && c->gbis_blocks > 0)
+  int rc;
+  if (c->gbis_blocks > 0) {
     rc = launch_rc(pa::launch_g_bisect_fused(c->g, c->pops, t, c->gbt, c->gbt + 3 * (size_t)pa::kGTableWeights,
-                                             c->gbar, c->gbis, target, 64, c->gbis_blocks, c->gbis_withheld,
+                                             c->gbar, c->gbis, rem, target, 64, c->gbis_blocks, c->gbis_withheld,
                                              c->stream));
-  else if (rc == PA_OK)
-    rc = launch_rc(pa::launch_g_bisect(c->g, c->pops, t, c->gw, c->gbis, target, 64, c->stream));
-  if (rc == PA_OK) rc = copy_d2h(c, b, c->gbis, sizeof b);
-  if (rc != PA_OK) return rc;
-  if (b[3] < 0.0) return PA_ERR_TIMEOUT;
+    if (rc == PA_OK) rc = copy_d2h(c, b, c->gbis, sizeof b);
+    if (rc != PA_OK) return rc;
+    if (b[3] < 0.0) return PA_ERR_TIMEOUT;
+    if (b[3] == 2.0) {
+      *dbeta = rem;
+      return PA_OK;
+    }
+  } else {
+    rc = copy_h2d(c, c->gbis, b, sizeof b);
+    if (rc == PA_OK) rc = launch_rc(pa::launch_g_tables(c->gbis + 2, 0.0, c->gw, c->stream));
+    if (rc == PA_OK) rc = launch_rc(pa::launch_g_eps_trial(c->g, c->pops, t, c->gw, c->stream));
+    double e = 0.0;
+    if (rc == PA_OK) rc = copy_d2h(c, &e, &c->pops[0].rec[t].eps_expected, sizeof(double));
+    if (rc != PA_OK) return rc;
+    if (e <= target) {
+      *dbeta = rem;
+      return PA_OK;
+    }
+    b[2] = 0.5 * (b[0] + b[1]);
+    rc = copy_h2d(c, c->gbis, b, sizeof b);
+    if (rc == PA_OK) rc = launch_rc(pa::launch_g_bisect(c->g, c->pops, t, c->gw, c->gbis, target, 64, c->stream));
+    if (rc == PA_OK) rc = copy_d2h(c, b, c->gbis, sizeof b);
+    if (rc != PA_OK) return rc;
+  }
   *dbeta = b[0] > 0.0 ? b[0] : b[1];
   return PA_OK;
 }
@@ -1271,7 +1279,7 @@ int pa_step(pa_ctx* c) try {
     // this step's site tables for the beta just chosen, built while the device resamples
     if (c->adaptive && rc == PA_OK) rc = upload_site_tables(c, c->betas[(size_t)t]);
     if (rc == PA_OK) {
-      PhaseTimer pt(c, PA_PHASE_SWEEP, 1);
+      PhaseTimer pt(c, PA_PHASE_SWEEP, 1 + c->g.n_pop);
       rc = launch_rc(pa::launch_g_sweep(c->g, c->pops, c->cur, c->jtab, c->Jq, c->Jtot,
                                         c->gtab + slot * c->g.N * pa::kGPatterns, t, c->sweeps[(size_t)t], s));
     }
