@@ -256,6 +256,44 @@ __global__ void __launch_bounds__(kCountThreads) k_g_counts(RunGeom g, GArgs a, 
   }
 }
 
+// ---------------------------------------------------------------- acceptance tables
+
+// One thread per site and pattern: min(floor(2^32 exp(-beta dE)), 2^32 - 2), 0xFFFFFFFF
+// for dE <= 0.  An entry with an integer within 2^-50 of v = 2^32 exp(-beta dE), relative
+// (at least four units in v's last place), is listed for the host: exponentials that
+// differ in their last bit could floor to different integers there.  (Building a step's
+// tables on eight host threads took 0.6 ms at L = 10, and all 60 tables of an L = 8
+// schedule, with a weight table for each, 45 of a run's 97 ms; the device idled.)
+__global__ void __launch_bounds__(256) k_g_site_tables(int L, const int32_t* __restrict__ Jq, double beta,
+                                                      uint32_t* gtab, int table, uint32_t* open) {
+  const int e = blockIdx.x * 256 + threadIdx.x, N = L * L * L;
+  if (e >= N * kGPatterns) return;
+  const int n = e / kGPatterns, b = e % kGPatterns;
+  const int x = n % L, y = (n / L) % L, z = n / (L * L);
+  const int xm = (x == 0 ? L - 1 : x - 1) + L * (y + L * z);
+  const int ym = x + L * ((y == 0 ? L - 1 : y - 1) + L * z);
+  const int zm = x + L * (y + L * (z == 0 ? L - 1 : z - 1));
+  const int bond[6] = {Jq[3 * n], Jq[3 * xm], Jq[3 * n + 1], Jq[3 * ym + 1], Jq[3 * n + 2], Jq[3 * zm + 2]};
+  int dE = 0;  // |dE| <= 2 * 6 * 5 * 2^20 < 2^31
+#pragma unroll
+  for (int k = 0; k < 6; ++k) dE += ((b >> k) & 1) ? -2 * bond[k] : 2 * bond[k];
+  uint32_t thr = 0xFFFFFFFFu;
+  if (dE > 0) {
+    const double v = __dmul_rn(exp(-__dmul_rn(beta, __dmul_rn((double)dE, 0x1p-20))), 4294967296.0);
+    const double tol = __dmul_rn(v, 0x1p-50);
+    const double lo = fmin(floor(__dsub_rn(v, tol)), 4294967294.0), hi = fmin(floor(__dadd_rn(v, tol)), 4294967294.0);
+    thr = (uint32_t)lo;
+    if (lo != hi) {
+      const uint32_t i = atomicAdd(&open[0], 1u);
+      if (i < (uint32_t)kGOpenCap) {
+        open[1 + 2 * i] = (uint32_t)table;
+        open[2 + 2 * i] = (uint32_t)e;
+      }
+    }
+  }
+  gtab[e] = thr;
+}
+
 // ---------------------------------------------------------------- adaptive schedule
 
 // Weight tables T_k[m] = exp(-dbeta m 2^(12k) 2^-20) (T0 | T1 | T2, kGTableWeights
@@ -828,6 +866,14 @@ __global__ void __launch_bounds__(kLinkThreads) k_g_link(RunGeom g, GArgs a, int
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
+
+int launch_g_site_tables(const RunGeom& g, const int32_t* Jq, double beta, uint32_t* gtab, int table, uint32_t* open,
+                         void* stream) {
+  const int per = g.N * kGPatterns;
+  k_g_site_tables<<<blocks_for(per, 256), 256, 0, (cudaStream_t)stream>>>(g.L, Jq, beta, gtab + (size_t)table * per,
+                                                                          table, open);
+  return (int)cudaGetLastError();
+}
 
 int launch_g_resample(const RunGeom& g, PopDev* pops, int cur, int t, const double* wtab, int32_t* status,
                       void* stream) {

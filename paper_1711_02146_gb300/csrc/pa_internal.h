@@ -193,6 +193,15 @@ int launch_family_hist(const RunGeom& g, PopDev* pops, int pop, int cur, int t, 
 int launch_scan_scatter(const RunGeom& g, PopDev* pops, int cur, int t, int32_t* status, void* stream);
 int launch_g_resample(const RunGeom& g, PopDev* pops, int cur, int t, const double* wtab, int32_t* status,
                       void* stream);
+// The acceptance tables of beta into table `table` of gtab ([N][kGPatterns] thresholds
+// each).  An entry whose floor could come out otherwise with another rounding of the
+// exponential (both this one and the C library's are within an ulp) is appended to the
+// list open = {length, entries}, two words per entry: its table, and site kGPatterns +
+// pattern; at most kGOpenCap entries are stored, the length counts all.
+constexpr int kGOpenCap = 127;
+constexpr int kGOpenWords = 1 + 2 * kGOpenCap;
+int launch_g_site_tables(const RunGeom& g, const int32_t* Jq, double beta, uint32_t* gtab, int table, uint32_t* open,
+                         void* stream);
 int launch_g_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
                    const uint32_t* gtab, int t, int n_sweeps, void* stream);
 // Step 0: the energies of the initial population in spins[1], which moves to spins[0].

@@ -18,8 +18,6 @@
 #include <memory>
 #include <mutex>
 #include <new>
-#include <system_error>
-#include <thread>
 #include <vector>
 
 #include "../../include/pa.h"
@@ -50,7 +48,8 @@ struct pa_ctx {
   std::vector<double> wtables_host;  // host copy of the explicit schedule's tables (source of their upload)
   double* wadapt = nullptr;     // adaptive schedule: the table of the current step
   double* wadapt_host = nullptr;  // its pinned host copy (uploaded without a wait)
-  uint32_t* gtab_host = nullptr;  // pinned host copy of the adaptive Gaussian step's site tables
+  uint32_t* gopen_host = nullptr;  // pinned: the site-table entries the device leaves open, and their values
+  std::vector<int32_t> gw_slot;    // explicit Gaussian schedule: the weight table (in gw) of each step
   int32_t occ_span = -1;          // adaptive +-1: highest minus lowest occupied level of population 0
   // All device buffers of the run are carved from one stream-ordered allocation:
   // a run costs the memory pool one block, so the pool's free list stays short
@@ -86,6 +85,7 @@ struct pa_ctx {
   cudaEvent_t step_ev[4] = {};
   int32_t step_ev_t[4] = {-1, -1, -1, -1};
   cudaStream_t rd = nullptr;
+  cudaEvent_t gopen_ev = nullptr;  // adaptive Gaussian step: the list of open site-table entries is on the host
 };
 
 namespace {
@@ -371,85 +371,79 @@ void gauss_couplings(int L, uint64_t seed, std::vector<int32_t>& Jq) {
   }
 }
 
-// Acceptance tables of one step: site n, pattern b of its bonds x+1, x-1, y+1,
-// y-1, z+1, z-1 (bit k set: bond k antiparallel), dE = 2 sum_k J_k (1 - 2 b_k):
-// the flip's Metropolis threshold, 0xFFFFFFFF for dE <= 0 (always taken), else
-// min(floor(2^32 exp(-beta dE 2^-20)), 2^32 - 2) in double precision.
-void gauss_site_tables_range(const std::vector<int32_t>& Jq, int L, double beta, uint32_t* out, int n0, int n1) {
-  for (int n = n0; n < n1; ++n) {
-    const int x = n % L, y = (n / L) % L, z = n / (L * L);
-    const int xm = (x == 0 ? L - 1 : x - 1) + L * (y + L * z);
-    const int ym = x + L * ((y == 0 ? L - 1 : y - 1) + L * z);
-    const int zm = x + L * (y + L * (z == 0 ? L - 1 : z - 1));
-    const int64_t bond[6] = {Jq[(size_t)3 * n + 0], Jq[(size_t)3 * xm + 0], Jq[(size_t)3 * n + 1],
-                             Jq[(size_t)3 * ym + 1], Jq[(size_t)3 * n + 2], Jq[(size_t)3 * zm + 2]};
-    for (int b = 0; b < pa::kGPatterns; ++b) {
-      int64_t dE = 0;  // flipping s_n: +2J for a parallel neighbour, -2J for an antiparallel one
-      for (int k = 0; k < 6; ++k) dE += bond[k] * (((b >> k) & 1) ? -1 : 1);
-      dE *= 2;
-      uint32_t thr = 0xFFFFFFFFu;
-      if (dE > 0) {
-        double v = std::floor(std::exp(-(beta * ((double)dE * 0x1p-20))) * 4294967296.0);
-        if (v > 4294967294.0) v = 4294967294.0;
-        thr = (uint32_t)v;
-      }
-      out[(size_t)n * pa::kGPatterns + b] = thr;
-    }
-  }
+// Acceptance tables of a step: site n, pattern b of its bonds x+1, x-1, y+1, y-1,
+// z+1, z-1 (bit k set: bond k antiparallel), dE = 2 sum_k J_k (1 - 2 b_k): the flip's
+// Metropolis threshold, 0xFFFFFFFF for dE <= 0 (always taken), else
+// min(floor(2^32 exp(-beta dE 2^-20)), 2^32 - 2) with the exponential rounded as the C
+// library rounds it.  The device builds them (launch_g_site_tables) and lists the few
+// entries whose floor the last bits of the exponential decide (some 1e-6 of them); those
+// are evaluated here.
+uint32_t site_threshold(const std::vector<int32_t>& Jq, int L, double beta, int n, int b) {
+  const int x = n % L, y = (n / L) % L, z = n / (L * L);
+  const int xm = (x == 0 ? L - 1 : x - 1) + L * (y + L * z);
+  const int ym = x + L * ((y == 0 ? L - 1 : y - 1) + L * z);
+  const int zm = x + L * (y + L * (z == 0 ? L - 1 : z - 1));
+  const int64_t bond[6] = {Jq[(size_t)3 * n + 0], Jq[(size_t)3 * xm + 0], Jq[(size_t)3 * n + 1],
+                           Jq[(size_t)3 * ym + 1], Jq[(size_t)3 * n + 2], Jq[(size_t)3 * zm + 2]};
+  int64_t dE = 0;  // flipping s_n: +2J for a parallel neighbour, -2J for an antiparallel one
+  for (int k = 0; k < 6; ++k) dE += bond[k] * (((b >> k) & 1) ? -1 : 1);
+  dE *= 2;
+  if (dE <= 0) return 0xFFFFFFFFu;
+  const double v = std::floor(std::exp(-(beta * ((double)dE * 0x1p-20))) * 4294967296.0);
+  return v > 4294967294.0 ? 0xFFFFFFFEu : (uint32_t)v;
 }
 
-// The site tables of all N sites; a large lattice's sites are split over a few
-// host threads (each entry is a function of its site alone, so the table is the same).
-void gauss_site_tables(const std::vector<int32_t>& Jq, int L, double beta, uint32_t* out) {
-  const int N = L * L * L;
-  const int n_thr = N < 512 ? 1 : (int)std::min<unsigned>(8u, std::max(1u, std::thread::hardware_concurrency()));
-  if (n_thr == 1) {
-    gauss_site_tables_range(Jq, L, beta, out, 0, N);
-    return;
-  }
-  std::vector<std::thread> pool;
-  pool.reserve((size_t)n_thr);
-  const int per = (N + n_thr - 1) / n_thr;
-  for (int k = 1; k < n_thr && k * per < N; ++k) {
-    const int a = k * per, b = std::min(N, (k + 1) * per);
-    try {
-      pool.emplace_back(gauss_site_tables_range, std::cref(Jq), L, beta, out, a, b);
-    } catch (const std::system_error&) {  // no thread to be had: this range here
-      gauss_site_tables_range(Jq, L, beta, out, a, b);
-    }
-  }
-  gauss_site_tables_range(Jq, L, beta, out, 0, std::min(N, per));
-  for (std::thread& th : pool) th.join();
+// The device list of open entries, kept behind the sweep's tables in the scratch of
+// population 0's buffer buf (PopDev).
+uint32_t* open_entries(const pa_ctx* c, int buf) {
+  const RunGeom& g = c->g;
+  return c->pops[0].spins[buf] + (size_t)g.pitch * g.sw + (size_t)g.N * pa::kGPatterns +
+         (size_t)g.N / 2 * pa::kGPatterns;
 }
 
-// Uploads the adaptive Gaussian step's site tables for beta, built into a pinned
-// buffer and copied without a wait (plain copy where pinned memory is not had).
-// The previous step's copy from that buffer is done: the bisection that chose beta
-// synchronised the stream.
-int upload_site_tables(pa_ctx* c, double beta) {
-  const size_t n = (size_t)c->g.N * pa::kGPatterns;
-  if (!c->gtab_host) {
+// Pinned host memory for that list and for the entries' values (null where none is had).
+uint32_t* pinned_entries(pa_ctx* c) {
+  if (!c->gopen_host) {
     void* h = nullptr;
-    if (cudaMallocHost(&h, sizeof(uint32_t) * n) == cudaSuccess)
-      c->gtab_host = static_cast<uint32_t*>(h);
+    if (cudaMallocHost(&h, sizeof(uint32_t) * (pa::kGOpenWords + pa::kGOpenCap)) == cudaSuccess)
+      c->gopen_host = static_cast<uint32_t*>(h);
     else
       cudaGetLastError();
   }
-  if (!c->gtab_host) {
-    std::vector<uint32_t> tab(n);
-    gauss_site_tables(c->Jq_host, c->g.L, beta, tab.data());
-    return copy_h2d(c, c->gtab, tab.data(), sizeof(uint32_t) * n);
-  }
-  gauss_site_tables(c->Jq_host, c->g.L, beta, c->gtab_host);
-  return copy_async(c, c->gtab, c->gtab_host, sizeof(uint32_t) * n);
+  return c->gopen_host;
 }
 
-// Weight tables of one step: T0[m] = exp(-dbeta m 2^-20), T1[m] for m 2^12,
-// T2[m] for m 2^24 (8192 entries).
-void gauss_weight_tables(double dbeta, double* T) {
+// Evaluates the listed entries (list[0] of them) of the tables of betas[first], betas[first
+// + 1], ... on the host and sends them to gtab, stream-ordered; values: kGOpenCap words
+// that stay alive until then.  A list that overflowed sends whole tables.
+int close_entries(pa_ctx* c, const uint32_t* list, uint32_t* values, const double* betas, size_t n_tables) {
+  const size_t per = (size_t)c->g.N * pa::kGPatterns;
+  int rc = PA_OK;
+  if (list[0] > (uint32_t)pa::kGOpenCap) {
+    std::vector<uint32_t> tab(per);
+    for (size_t k = 0; k < n_tables && rc == PA_OK; ++k) {
+      for (size_t e = 0; e < per; ++e)
+        tab[e] = site_threshold(c->Jq_host, c->g.L, betas[k], (int)(e / pa::kGPatterns), (int)(e % pa::kGPatterns));
+      rc = copy_h2d(c, c->gtab + k * per, tab.data(), sizeof(uint32_t) * per);
+    }
+    return rc;
+  }
+  for (uint32_t i = 0; i < list[0] && rc == PA_OK; ++i) {
+    const size_t k = list[1 + 2 * i], e = list[2 + 2 * i];
+    values[i] = site_threshold(c->Jq_host, c->g.L, betas[k], (int)(e / pa::kGPatterns), (int)(e % pa::kGPatterns));
+    rc = copy_async(c, c->gtab + k * per + e, values + i, sizeof(uint32_t));
+  }
+  return rc;
+}
+
+// Weight tables of an increment: T0[m] = exp(-dbeta m 2^-20), T1[m] for m 2^12, T2[m] for
+// m 2^24, T2 up to the largest energy difference of a lattice of N sites (couplings are
+// clamped to 5: |E| <= 15 N).
+void gauss_weight_tables(int N, double dbeta, double* T) {
+  const int n2 = std::min(8192, 30 * N / 16 + 2);
   for (int m = 0; m < 4096; ++m) T[m] = std::exp(-(dbeta * ((double)m * 0x1p-20)));
   for (int m = 0; m < 4096; ++m) T[4096 + m] = std::exp(-(dbeta * ((double)((int64_t)m << 12) * 0x1p-20)));
-  for (int m = 0; m < 8192; ++m) T[8192 + m] = std::exp(-(dbeta * ((double)((int64_t)m << 24) * 0x1p-20)));
+  for (int m = 0; m < n2; ++m) T[8192 + m] = std::exp(-(dbeta * ((double)((int64_t)m << 24) * 0x1p-20)));
 }
 
 uint64_t bits_of(double x) {
@@ -737,9 +731,10 @@ void destroy(pa_ctx* c) {
   for (cudaEvent_t e : c->events) cudaEventDestroy(e);
   for (cudaEvent_t e : c->step_ev)
     if (e) cudaEventDestroy(e);
+  if (c->gopen_ev) cudaEventDestroy(c->gopen_ev);
   if (c->rd) cudaStreamDestroy(c->rd);
   if (c->wadapt_host) cudaFreeHost(c->wadapt_host);
-  if (c->gtab_host) cudaFreeHost(c->gtab_host);
+  if (c->gopen_host) cudaFreeHost(c->gopen_host);
   delete c;
 }
 
@@ -1182,23 +1177,29 @@ int create_run_impl(const pa_config* cfg, void* cuda_stream, pa_ctx** out, bool 
   // Host tables go up in one copy per kind; the +-1 tables' host buffer lives in
   // the run, the Gaussian ones until the stream synchronisation at the end of
   // creation (always taken for that model).
-  std::vector<uint32_t> gtab_all;
   std::vector<double> gw_all;
   if (g.model == PA_MODEL_GAUSS) {
     // couplings, and the acceptance and weight tables of every step, on the host
     gauss_couplings(g.L, cfg->disorder_seed, c->Jq_host);
     for (int32_t v : c->Jq_host) c->Jtot += v;
     if (rc == PA_OK) rc = copy_async(c, c->Jq, c->Jq_host.data(), sizeof(int32_t) * c->Jq_host.size());
-    if (!c->adaptive && T > 1) {
-      const size_t per_tab = (size_t)g.N * pa::kGPatterns;
-      gtab_all.assign(T * per_tab, 0u);
-      gw_all.assign(T * (size_t)pa::kGTableWeights, 0.0);
-      for (size_t t = 1; t < T; ++t) {
-        gauss_site_tables(c->Jq_host, g.L, c->betas[t], gtab_all.data() + t * per_tab);
-        gauss_weight_tables(c->betas[t] - c->betas[t - 1], gw_all.data() + t * (size_t)pa::kGTableWeights);
-      }
-      if (rc == PA_OK) rc = copy_async(c, c->gtab, gtab_all.data(), sizeof(uint32_t) * gtab_all.size());
+    if (!c->adaptive && T > 1) {  // one weight table per distinct increment, one site table per step
+      const std::vector<double> d = distinct_dbetas(c->betas);
+      gw_all.assign(d.size() * (size_t)pa::kGTableWeights, 0.0);
+      for (size_t i = 0; i < d.size(); ++i) gauss_weight_tables(g.N, d[i], gw_all.data() + i * (size_t)pa::kGTableWeights);
+      c->gw_slot.assign(T, 0);
+      for (size_t t = 1; t < T; ++t)
+        for (size_t i = 0; i < d.size(); ++i)
+          if (bits_of(d[i]) == bits_of(c->betas[t] - c->betas[t - 1])) c->gw_slot[t] = (int32_t)i;
       if (rc == PA_OK) rc = copy_async(c, c->gw, gw_all.data(), sizeof(double) * gw_all.size());
+      uint32_t* open = open_entries(c, 0);
+      std::vector<uint32_t> list(pa::kGOpenWords, 0u), values(pa::kGOpenCap);
+      if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(open, 0, sizeof(uint32_t), s));
+      for (size_t t = 1; t < T && rc == PA_OK; ++t)
+        rc = launch_rc(pa::launch_g_site_tables(g, c->Jq, c->betas[t], c->gtab, (int)t, open, s));
+      if (rc == PA_OK) rc = copy_d2h(c, list.data(), open, sizeof(uint32_t) * list.size());
+      if (rc == PA_OK) rc = close_entries(c, list.data(), values.data(), c->betas.data(), T);
+      if (rc == PA_OK && list[0]) rc = cuda_status(cudaStreamSynchronize(s));  // values leaves scope
     }
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->J, 0, (size_t)3 * g.N, s));
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->jtab, 0, sizeof(uint32_t) * 4 * g.N, s));
@@ -1268,16 +1269,40 @@ int pa_step(pa_ctx* c) try {
     rc = cuda_status(cudaMemsetAsync(c->pops[p].rec + t, 0, sizeof(StepRec), s));
   if (c->model == PA_MODEL_GAUSS) {
     const size_t slot = c->adaptive ? 0 : (size_t)t;
-    // the weight tables as the bisection's trials built them, so the resampling's
-    // culling fraction is the one the bisection accepted
-    if (c->adaptive && rc == PA_OK) rc = launch_rc(pa::launch_g_tables(nullptr, dbeta, c->gw, c->stream));
+    const size_t wslot = c->adaptive ? 0 : (size_t)c->gw_slot[(size_t)t];
+    // The weight tables as the bisection's trials built them, so the resampling's culling
+    // fraction is the one the bisection accepted, and the site tables of the beta just
+    // chosen; the host settles the entries that the device left open while it resamples.
+    uint32_t* open = open_entries(c, 1 - c->cur);
+    uint32_t* host = c->adaptive ? pinned_entries(c) : nullptr;
+    if (c->adaptive) {
+      if (rc == PA_OK) rc = launch_rc(pa::launch_g_tables(nullptr, dbeta, c->gw, c->stream));
+      if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(open, 0, sizeof(uint32_t), s));
+      if (rc == PA_OK) rc = launch_rc(pa::launch_g_site_tables(c->g, c->Jq, c->betas[(size_t)t], c->gtab, 0, open, s));
+      if (host && rc == PA_OK) {
+        c->stats.d2h_bytes += (int64_t)sizeof(uint32_t) * pa::kGOpenWords;
+        rc = cuda_status(cudaMemcpyAsync(host, open, sizeof(uint32_t) * pa::kGOpenWords, cudaMemcpyDeviceToHost, s));
+        if (rc == PA_OK && !c->gopen_ev) rc = cuda_status(cudaEventCreateWithFlags(&c->gopen_ev, cudaEventDisableTiming));
+        if (rc == PA_OK) rc = cuda_status(cudaEventRecord(c->gopen_ev, s));
+      }
+    }
     if (rc == PA_OK) {
       PhaseTimer pt(c, PA_PHASE_RESAMPLE, 7);
-      rc = launch_rc(pa::launch_g_resample(c->g, c->pops, c->cur, t, c->gw + slot * pa::kGTableWeights,
+      rc = launch_rc(pa::launch_g_resample(c->g, c->pops, c->cur, t, c->gw + wslot * pa::kGTableWeights,
                                            c->status, s));
     }
-    // this step's site tables for the beta just chosen, built while the device resamples
-    if (c->adaptive && rc == PA_OK) rc = upload_site_tables(c, c->betas[(size_t)t]);
+    if (c->adaptive && rc == PA_OK) {
+      const double beta = c->betas[(size_t)t];
+      if (host) {
+        rc = cuda_status(cudaEventSynchronize(c->gopen_ev));
+        if (rc == PA_OK) rc = close_entries(c, host, host + pa::kGOpenWords, &beta, 1);
+      } else {
+        std::vector<uint32_t> list(pa::kGOpenWords, 0u), values(pa::kGOpenCap);
+        rc = copy_d2h(c, list.data(), open, sizeof(uint32_t) * list.size());
+        if (rc == PA_OK) rc = close_entries(c, list.data(), values.data(), &beta, 1);
+        if (rc == PA_OK && list[0]) rc = cuda_status(cudaStreamSynchronize(s));  // values leaves scope
+      }
+    }
     if (rc == PA_OK) {
       PhaseTimer pt(c, PA_PHASE_SWEEP, 1 + c->g.n_pop);
       rc = launch_rc(pa::launch_g_sweep(c->g, c->pops, c->cur, c->jtab, c->Jq, c->Jtot,
