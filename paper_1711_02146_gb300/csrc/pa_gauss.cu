@@ -335,7 +335,7 @@ __global__ void k_g_tables(const double* __restrict__ dbeta_dev, double dbeta_va
 // therefore find a point below which every midpoint from dbeta0 on is accepted and one
 // above which every midpoint is rejected, each by more than the rounding of e (about
 // 1e-14; kTrialMargin), and only the midpoints between them (and below dbeta0) are tried.
-// That leaves some 25 of 58 trials; a trial takes about 20 us instead of 55 at R = 1e6
+// That leaves some 24 of 58 trials; a trial takes about 30 us instead of 55 at R = 1e6
 // (FP64 pipe: 7 operations per replica, 10 us).
 constexpr int kBisectThreads = 512;
 constexpr int kBisectWarps = kBisectThreads / 32;
@@ -373,25 +373,22 @@ __device__ double block_total(const double* part, int n, double* lvl) {
   return x;
 }
 
-// Grid barrier of a cooperative launch: the last block to arrive resets the count
-// and advances the generation, the others poll it at most `spins` times.  With
-// part, that last block first stores block_total(part, n) in bar[slot].  A wait that
-// runs out records the error, after which every barrier returns at once (false) and
-// the launch ends with the error set.  A block with withhold set waits without
-// arriving (a test of that path: the waits then run out).
-__device__ bool grid_barrier(unsigned long long* bar, unsigned spins_max, bool withhold = false,
+// Grid barrier number `round` (0, 1, ...) of a cooperative launch: the arrivals are
+// counted on through all barriers, the last block to arrive stores round + 1 as the
+// generation and the others poll it at most `spins` times.  With part, that last block
+// first stores block_total(part, n) in bar[slot].  A wait that runs out records the
+// error, after which every barrier returns at once (false) and the launch ends with the
+// error set.  A block with withhold set waits without arriving (a test of that path: the
+// waits then run out).
+__device__ bool grid_barrier(unsigned long long* bar, unsigned round, unsigned spins_max, bool withhold = false,
                              const double* part = nullptr, int n = 0, int slot = 0, double* lvl = nullptr) {
   __shared__ int state;  // 0: wait, 1: last to arrive, -1: error
   volatile unsigned long long* vb = bar;
-  unsigned long long gen = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
-    int st = vb[kBarError] == 0ull ? 0 : -1;
-    if (st == 0) {
-      gen = vb[kBarGen];
-      __threadfence();
-      if (!withhold && atomicAdd(&bar[kBarArrive], 1ull) == (unsigned long long)gridDim.x - 1ull) st = 1;
-    }
+    __threadfence();
+    int st = 0;
+    if (!withhold && atomicAdd(&bar[kBarArrive], 1ull) == (unsigned long long)gridDim.x * (round + 1ull) - 1ull) st = 1;
     state = st;
   }
   __syncthreads();
@@ -402,17 +399,18 @@ __device__ bool grid_barrier(unsigned long long* bar, unsigned spins_max, bool w
   if (threadIdx.x == 0) {
     if (state == 1) {
       __threadfence();
-      atomicExch(&bar[kBarArrive], 0ull);
-      __threadfence();
-      atomicAdd(&bar[kBarGen], 1ull);
-    } else if (state == 0) {
+      vb[kBarGen] = round + 1ull;
+    } else {
       unsigned spins = 0;
-      while (vb[kBarGen] == gen && vb[kBarError] == 0ull && ++spins < spins_max) __nanosleep(64);
-      if (vb[kBarGen] == gen) {
-        atomicExch(&bar[kBarError], 1ull);
-        state = -1;
+      while (vb[kBarGen] <= round && ++spins < spins_max) {
+        if (spins > 64u) {
+          if (vb[kBarError] != 0ull) break;
+          __nanosleep(64);
+        }
       }
+      if (vb[kBarGen] <= round) atomicExch(&bar[kBarError], 1ull);
     }
+    if (vb[kBarError] != 0ull) state = -1;
     __threadfence();
   }
   __syncthreads();
@@ -506,11 +504,12 @@ __global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
     dmax = x > dmax ? x : dmax;
   }
   if (lane == 0 && dmax) atomicMax(&a.bar[kBarDmax], dmax);
-  bool ok = grid_barrier(a.bar, a.spins, (int)blockIdx.x == a.withheld);
+  unsigned round = 0;  // barriers passed, the same in every block
+  bool ok = grid_barrier(a.bar, round++, a.spins, (int)blockIdx.x == a.withheld);
   const int n_tab = 8192 + (int)min(8191ull, ((volatile unsigned long long*)a.bar)[kBarDmax] >> 24) + 1;
 
-  auto build = [&](int set, double db) {  // this block's share of the tables of db
-    for (int m = gtid; m < n_tab; m += n_threads) __stcg(a.T + (size_t)set * kGTableWeights + m, g_table_entry(db, m));
+  auto build = [&](int set, double db) {  // this block's share of the tables of db, the blocks in turn
+    for (int m = (int)(blockIdx.x + gridDim.x * threadIdx.x); m < n_tab; m += n_threads) __stcg(a.T + (size_t)set * kGTableWeights + m, g_table_entry(db, m));
   };
   auto weight = [&](uint32_t lo, int hi) {
     return __dmul_rn(__dmul_rn(tab[8192 + hi], tab[4096 + (lo >> 12)]), tab[lo & 4095u]);
@@ -548,7 +547,7 @@ __global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
       const double sum = group8(v);
       if (lane == 0) __stcg(P.part + c, sum);
     }
-    if (!grid_barrier(a.bar, a.spins, false, P.part, nch, kBarS, lvl)) {
+    if (!grid_barrier(a.bar, round++, a.spins, false, P.part, nch, kBarS, lvl)) {
       ok = false;
       return 0.0;
     }
@@ -582,7 +581,7 @@ __global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
       const double sum = group8(v);
       if (lane == 0) __stcg(a.part1 + c, sum);
     }
-    if (!grid_barrier(a.bar, a.spins, false, a.part1, nch, kBarCull, lvl)) {
+    if (!grid_barrier(a.bar, round++, a.spins, false, a.part1, nch, kBarCull, lvl)) {
       ok = false;
       return 0.0;
     }
@@ -591,7 +590,7 @@ __global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
   auto nothing = [] {};
   auto trial_at = [&](double x) -> double {
     build(0, x);
-    if (!grid_barrier(a.bar, a.spins)) {
+    if (!grid_barrier(a.bar, round++, a.spins)) {
       ok = false;
       return 0.0;
     }
@@ -640,7 +639,7 @@ __global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
     int cur = 0;
     if (ok && !s.done) {
       build(cur, s.mid);
-      ok = grid_barrier(a.bar, a.spins);
+      ok = grid_barrier(a.bar, round++, a.spins);
     }
     while (ok && !s.done) {
       Halving acc = s, rej = s;
@@ -666,7 +665,7 @@ __global__ void __launch_bounds__(kBisectThreads, 1) k_g_bisect(BisectArgs a) {
         known.settle(s, a.halvings);
         if (!s.done && s.mid != mid) {
           build(cur, s.mid);
-          ok = grid_barrier(a.bar, a.spins);
+          ok = grid_barrier(a.bar, round++, a.spins);
         }
       }
     }
