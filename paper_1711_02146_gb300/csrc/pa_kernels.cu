@@ -146,9 +146,12 @@ __global__ void __launch_bounds__(256) k_copy_parents(RunGeom g, PopDev P, int c
 //   S' = sum_{k >= kmin} c(k) w[k - kmin]         (ascending k, separate mul/add)
 //   tau_k = R w[k - kmin] / S'  ->  fl_k = floor(tau_k), thr_k = 2^32 (tau_k - fl_k)
 //   eps = (1/R) sum_k c(k) (1 - tau_k)_+          (Eq. eq_num_elim; fixed tree order)
-// Empty levels add exact zeros to S', so they are skipped there.
+// Empty levels add exact zeros to S', so they are skipped there, and no slot reads
+// their tau, so they get none (a division for each of the 3N+1 levels took 11 of the
+// 29 us at L = 10 on GB300's narrow FP64 pipe; the occupied ones are some 200).
 // One block per population; lst_sh (n_levels entries) holds the occupied levels,
-// ascending, when list_in_smem.
+// ascending, when list_in_smem.  The rest is latency: the additions of S' in level order
+// (one after the other), a division, the barriers.
 __device__ __forceinline__ void reweight_pop(const RunGeom& g, const PopDev& P, const double* __restrict__ w, int t,
                                              int* lst_sh, int list_in_smem) {
   __shared__ int scratch[33];
@@ -158,17 +161,31 @@ __device__ __forceinline__ void reweight_pop(const RunGeom& g, const PopDev& P, 
   // which is only written (below) after the list has been read
   int* lst = list_in_smem ? lst_sh : P.fl;
   const uint32_t* c = P.hist + (size_t)(t - 1) * g.n_levels;
-  int base = 0;
-  for (int k0 = 0; k0 < g.n_levels; k0 += blockDim.x) {
-    const int k = k0 + threadIdx.x;
-    const int f = (k < g.n_levels && c[k] > 0u) ? 1 : 0;
-    int tot;
-    const int pos = block_exclusive_scan(f, scratch, &tot);
-    if (f) lst[base + pos] = k;
-    base += tot;
+  // each warp takes whole groups of 32 levels in a row: their occupied ones are counted,
+  // the counts scanned over the warps, and the list filled (one scan for any n_levels)
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int groups = (g.n_levels + 31) / 32, per = (groups + 31) / 32, g0 = warp * per, g1 = min(groups, g0 + per);
+  auto occupied = [&](int gr) {
+    const int k = 32 * gr + lane;
+    return __ballot_sync(0xffffffffu, k < g.n_levels && c[k] > 0u);
+  };
+  int mine = 0;
+  for (int gr = g0; gr < g1; ++gr) mine += __popc(occupied(gr));
+  if (lane == 0) scratch[warp] = mine;
+  __syncthreads();
+  if (warp == 0) {
+    const int v = scratch[lane], inc = warp_inclusive_scan(v);
+    scratch[lane] = inc - v;
+    if (lane == 31) scratch[32] = inc;
   }
   __syncthreads();
-  const int nnz = base;
+  for (int gr = g0, at = scratch[warp]; gr < g1; ++gr) {
+    const unsigned o = occupied(gr);
+    if ((o >> lane) & 1u) lst[at + __popc(o & ((1u << lane) - 1u))] = 32 * gr + lane;
+    at += __popc(o);
+  }
+  const int nnz = scratch[32];
+  __syncthreads();
   if (nnz == 0) return;  // cannot happen: the population is never empty here
   const int kmin = lst[0];
   // S' = the sum over occupied levels, ascending, of c(k) w(k - kmin): every thread
@@ -194,32 +211,36 @@ __device__ __forceinline__ void reweight_pop(const RunGeom& g, const PopDev& P, 
   const double S = S_sh;
   const double Rd = (double)g.R;
   double eps_part = 0.0;  // this thread's levels, ascending
-  for (int k = threadIdx.x; k < g.n_levels; k += blockDim.x) {
-    int f = 0;
-    uint32_t th = 0u;
-    if (k >= kmin) {
-      const double tau = __ddiv_rn(__dmul_rn(Rd, w[k - kmin]), S);
-      const double fl = floor(tau);
-      f = (int)fl;
-      th = (uint32_t)__dmul_rn(__dsub_rn(tau, fl), 4294967296.0);
-      if (tau < 1.0 && c[k] > 0u) eps_part = __dadd_rn(eps_part, __dmul_rn((double)c[k], __dsub_rn(1.0, tau)));
-    }
-    P.fl[k] = f;
-    P.thr[k] = th;
+  const int kmax = lst[nnz - 1];
+  __syncthreads();  // the list (in the floor table) has been read
+  for (int k = threadIdx.x; k <= kmax; k += blockDim.x) {
+    const uint32_t ck = c[k];
+    if (ck == 0u) continue;
+    const double tau = __ddiv_rn(__dmul_rn(Rd, w[k - kmin]), S);
+    const double fl = floor(tau);
+    P.fl[k] = (int)fl;
+    P.thr[k] = (uint32_t)__dmul_rn(__dsub_rn(tau, fl), 4294967296.0);
+    if (tau < 1.0) eps_part = __dadd_rn(eps_part, __dmul_rn((double)ck, __dsub_rn(1.0, tau)));
   }
   // expected culling fraction (Eq. eq_num_elim / R): fixed tree over the threads
   eps_sh[threadIdx.x] = eps_part;
   __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
+  for (int h = blockDim.x / 2; h >= 32; h >>= 1) {
     if ((int)threadIdx.x < h) eps_sh[threadIdx.x] = __dadd_rn(eps_sh[threadIdx.x], eps_sh[threadIdx.x + h]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    StepRec& r = P.rec[t];
-    r.S_prime = S;
-    r.eps_expected = __ddiv_rn(eps_sh[0], Rd);
-    r.kmin_prev = kmin;
-    r.R_prev = P.rec[t - 1].R_tilde;
+  if (warp == 0) {
+    double e = eps_sh[lane];
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) e = __dadd_rn(e, __shfl_down_sync(0xffffffffu, e, h));
+    if (lane == 0) {
+      StepRec r{};
+      r.S_prime = S;
+      r.eps_expected = __ddiv_rn(e, Rd);
+      r.kmin_prev = kmin;
+      r.R_prev = P.rec[t - 1].R_tilde;
+      P.rec[t] = r;  // opens the step's record; the later kernels add to it
+    }
   }
 }
 
@@ -228,14 +249,12 @@ __global__ void k_reweight(RunGeom g, PopArgs a, const double* __restrict__ w, i
   reweight_pop(g, a.p[blockIdx.x], w, t, lst_sh, list_in_smem);
 }
 
-// Every unit of a batch, one block each; the step record of the round's step is
-// cleared here (a lone run clears it with a memset before this kernel).
+// Every unit of a batch, one block each.
 __global__ void k_group_reweight(const GroupUnit* __restrict__ units, const int32_t* __restrict__ round) {
   extern __shared__ int lst_sh[];
   const GroupUnit& u = units[blockIdx.x];
   const int t = u.t0 + 1 + *round;
   if (t > u.last_t) return;
-  if (threadIdx.x == 0) u.P.rec[t] = StepRec{};
   reweight_pop(u.g, u.P, u.steps[t].w, t, lst_sh, 1);
 }
 

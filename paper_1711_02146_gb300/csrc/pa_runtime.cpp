@@ -1265,7 +1265,7 @@ int pa_step(pa_ctx* c) try {
   }
   cudaStream_t s = c->stream;
   int rc = PA_OK;
-  for (int p = 0; p < c->g.n_pop && rc == PA_OK; ++p)
+  for (int p = 0; p < c->g.n_pop && rc == PA_OK && c->model == PA_MODEL_GAUSS; ++p)  // +-1: the reweighting does
     rc = cuda_status(cudaMemsetAsync(c->pops[p].rec + t, 0, sizeof(StepRec), s));
   if (c->model == PA_MODEL_GAUSS) {
     const size_t slot = c->adaptive ? 0 : (size_t)t;
@@ -2340,7 +2340,6 @@ int pa_shard_step(pa_shard* s) try {
   const double dbeta = c->betas[(size_t)t] - c->betas[(size_t)t - 1];
   cudaStream_t st = c->stream;
   int rc = PA_OK;
-  for (int p = 0; p < np && rc == PA_OK; ++p) rc = cuda_status(cudaMemsetAsync(c->pops[p].rec + t, 0, sizeof(StepRec), st));
   // 1-2. tables from the global histogram of step t-1; copy numbers of the local old
   // slots (their uniforms addressed by global slot) and the copies in local order
   const double* w = nullptr;
