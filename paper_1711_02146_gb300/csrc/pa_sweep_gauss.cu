@@ -286,9 +286,13 @@ __global__ void __launch_bounds__(NT, MB) k_sweep_g(const __grid_constant__ GSwe
   constexpr int N = S::N, NP = S::NP, TJ = S::TJ;
   const SweepArgs& a = ga.base;
   extern __shared__ __align__(1024) uint32_t smg[];
+  launch_dependents();
   const int R_new = a.pop.rec[a.t].R_tilde;
   const int tile0 = blockIdx.x * TJ;
-  if (tile0 >= R_new) return;
+  if (tile0 >= R_new) {
+    wait_launch_before((R_new + TJ - 1) / TJ);
+    return;
+  }
   uint32_t* sp = smg + S::TABLES / 4;
   uint2* phil = reinterpret_cast<uint2*>(sp + (size_t)N * W);
   int* elo = reinterpret_cast<int*>(phil + N);
@@ -336,6 +340,7 @@ __global__ void __launch_bounds__(NT, MB) k_sweep_g(const __grid_constant__ GSwe
   __syncthreads();  // the energies are read before the rows take their place
   store_bits<S>(a, sp, tile0);
   store_done<RowMove<S>>();
+  wait_launch_before((R_new + TJ - 1) / TJ);
 }
 
 template <int L, int W, int NT, int MB>
@@ -344,9 +349,8 @@ int launch_g_t(const RunGeom& g, const GSweepArgs& args, cudaStream_t s) {
   static std::atomic<int> done[64];
   const cudaError_t e = smem_limit_once(k_sweep_g<L, W, NT, MB>, (int)S::SMEM, done);
   if (e != cudaSuccess) return (int)e;
-  dim3 grid((unsigned)((g.R_cap + S::TJ - 1) / S::TJ));
-  k_sweep_g<L, W, NT, MB><<<grid, NT, S::SMEM, s>>>(args);
-  return (int)cudaGetLastError();
+  const unsigned grid = (unsigned)((g.R_cap + S::TJ - 1) / S::TJ);
+  return launch_tiles(k_sweep_g<L, W, NT, MB>, grid, NT, S::SMEM, args.base, args, s);
 }
 
 int g_sweep_launches(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
@@ -373,6 +377,7 @@ int g_sweep_launches(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jt
     args.tile_base = 0;
     args.split = 0x7fffffff;
     args.tj_main = args.tj_tail = 1;
+    args.chained = i > 0 ? 1 : 0;
     ga.gtab = gtab;
     ga.utab = utab;
     ga.etab = etab;
