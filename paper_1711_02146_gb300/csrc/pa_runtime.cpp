@@ -941,6 +941,19 @@ T read_at(const char* p, size_t i) {
   return v;
 }
 
+// Whether all n bytes are spins (0x01 or 0xFF), eight at a time (n is a multiple of N, and
+// N = L^3 of eight): with its lowest bit flipped a spin's bits are all 0 (+1) or 0 and
+// seven 1s (-1).  A byte at a time, with an exit in the loop, it took 8 of the 13 ms of a
+// restore of 5e4 replicas of L = 8; saving and resuming them 18.1 -> 10.5 ms.
+bool all_spins(const char* in, size_t n) {
+  uint64_t bad = 0;
+  for (size_t i = 0; i < n / 8; ++i) {
+    const uint64_t y = read_at<uint64_t>(in, i) ^ 0x0101010101010101ull;
+    bad |= (y & 0x0101010101010101ull) | ((y ^ (y >> 1)) & 0x7E7E7E7E7E7E7E7Eull);
+  }
+  return bad == 0;
+}
+
 // Checks the population part of a checkpoint on the host, before any of it
 // reaches the device: every value a kernel later uses as an index or a size must
 // be in range and consistent.  Step records chain (each step's previous size is
@@ -983,10 +996,7 @@ bool ckpt_payload_ok(const RunGeom& g, bool gauss, int t, int64_t R, const CkptH
       in += sizeof(uint32_t) * ((size_t)t + 1) * (size_t)g.n_levels;
     }
     const size_t n_spins = (size_t)g.N * (size_t)Rt;
-    for (size_t i = 0; i < n_spins; ++i) {
-      const uint8_t b = (uint8_t)in[i];
-      if (b != 0x01 && b != 0xFF) return false;
-    }
+    if (!all_spins(in, n_spins)) return false;
     in += n_spins;
     for (int64_t j = 0; j < Rt; ++j) {
       const int32_t l = read_at<int32_t>(in, (size_t)j);
