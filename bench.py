@@ -7,7 +7,7 @@ glass, L = 10 (1000 sites), R = 10^6 replicas, temperature steps chosen to hold
 the culling fraction at 0.272 up to beta = 5, 10 sweeps per step.  A "step" is
 one temperature step of the whole hot path: reweight, copy numbers + scan +
 parents, parent gather + 10 Metropolis sweeps + energy levels/histogram, family
-statistics.  The 2 GB double-buffered population is far larger than L2, so no
+statistics.  The population (a bit per spin, two buffers in turn: 256 MB) is larger than L2, so no
 flush is needed between steps.
 
 value   = Metropolis site updates (sum over timed steps of S N R~_t) / device time
@@ -54,12 +54,13 @@ UNIT = "updates/s"
 # The work of one update (integer instructions per update, ncu) and the rate are
 # read from each kernel's committed profile summary.
 # HBM bytes per update of the sweep kernel: the tile is read (gather) and
-# written once per step, i.e. 2 bytes per site and replica every S sweeps, plus
+# written once per step, i.e. 2 bits per site and replica every S sweeps, plus
 # 8 bytes of parent index and energy level per replica.
 
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "sweep_L10_R1e6_adaptive.txt")
 GAUSS_PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "sweep_gauss_L10_R1e6_linear101.txt")
-SWEEP_SOURCE = os.path.join(ROOT, "paper_1711_02146_gb300", "csrc", "pa_sweep.cu")
+SWEEP_SOURCES = [os.path.join(ROOT, "paper_1711_02146_gb300", "csrc", f) for f in
+                 ("pa_bits.cuh", "pa_metropolis.cuh", "pa_sweep_tile.cuh", "pa_sweep_gauss.cu", "pa_sweep_l10.cu")]
 
 
 def parse():
@@ -311,7 +312,7 @@ def profile_lines(path: str):
 
 
 def source_digest() -> str:
-    return hashlib.sha256(open(SWEEP_SOURCE, "rb").read()).hexdigest()[:16]
+    return hashlib.sha256(b"".join(open(f, "rb").read() for f in SWEEP_SOURCES)).hexdigest()[:16]
 
 
 def tail_kernel(L: int, tail):
@@ -707,7 +708,7 @@ def ours(args):
     if traffic is not None:
         traffic = traffic * updates_per_launch / (w.n_sweeps * w.N * w.R)
     replicas = updates_per_launch / (w.n_sweeps * w.N)
-    hbm_bytes = 2.0 * w.N * replicas + 8.0 * replicas
+    hbm_bytes = 2.0 * w.N / 8.0 * replicas + 8.0 * replicas
     hbm_peak = measured_hbm_gbs()
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gupdates/s",
                 "frac": achieved / peak if peak else None, "traffic": traffic,
@@ -741,7 +742,7 @@ def ours(args):
             "config": {"workload": w.name, "L": w.L, "R": w.R, "eps_target": w.eps_target, "beta_max": w.beta_max,
                        "n_sweeps": w.n_sweeps, "steps_timed": f"temperature steps {args.warmup + 1}.."
                                                               f"{args.warmup + done}",
-                       "l2": "inputs larger than L2 (2 GB double-buffered int8 population)",
+                       "l2": "inputs larger than L2 (population of one bit per spin in two buffers, 256 MB in all)",
                        "sweep_shapes": tuned},
             "roofline": roofline, "resample": resample, "e2e": e2e, "gpu_launches": st["kernel_launches"],
             "phase_share": phase_share, "clocks": clk}
