@@ -1,5 +1,6 @@
 // pa_gauss.cu — the Gaussian-coupling model (§II.A: J ~ N(0,1)):
-// resampling from per-replica weights, energy moments and the link overlap.  (Its sweep kernel, k_sweep_g, lives with the other sweep kernels.)
+// resampling from per-replica weights, energy moments and the link overlap (its sweep
+// kernel, k_sweep_g, is in pa_sweep_gauss.cu).
 //
 // Couplings and energies are fixed point (units of 2^-20, couplings clamped to
 // [-5, 5]), so energies, their sums and the link overlap are exact integers and

@@ -2,7 +2,7 @@
 // (§II.A), in the tiles of the +-1 kernel (pa_sweep_tile.cuh): one bit per replica, 32
 // replicas per word, N sites, rows staged through shared memory.
 //
-// The acceptance comes from a per-site table built on the host for the step's beta: for
+// The acceptance comes from a per-site table (k_g_site_tables) for the step's beta: for
 // each of the 64 patterns of antiparallel neighbours (bit k: bond k, in the order x+1,
 // x-1, y+1, y-1, z+1, z-1) the threshold of the flip, 0xFFFFFFFF when it costs dE <= 0
 // (always taken) and otherwise min(floor(2^32 exp(-beta dE)), 2^32 - 2); the flip is

@@ -101,8 +101,7 @@ __device__ __forceinline__ void fill_row_table(int* rowtab, int tid, int nthread
   }
 }
 
-// ---- phases of a tile: init_tables and publish_levels serve both kernels,
-// gather_tile and store_tile are the Gaussian kernel's (nibble tiles)
+// ---- phases of a tile
 
 // Site records (bond masks, site/step parts of Philox rounds 1-3); all
 // `nthreads` threads of the CTA help.
