@@ -220,6 +220,12 @@ int pa_get_genergies(pa_ctx* ctx, int32_t pop, int64_t first, int64_t n, int64_t
 int pa_ql_hist(pa_ctx* ctx, int32_t t, int64_t* out, int64_t cap);
 /* Fixed-point couplings Jq[3n + d] (3N int32, units of 2^-20) of a Gaussian run. */
 int pa_get_gcouplings(pa_ctx* ctx, int32_t* Jq, int64_t cap);
+/* Metropolis thresholds of step t >= 1 (cap >= 64 N entries), entry 64 n + b for site n
+ * and pattern b of its antiparallel neighbours (bit k: bond k, in the order x+1, x-1,
+ * y+1, y-1, z+1, z-1): 2^32 - 1 where the flip costs dE <= 0 (always taken), else
+ * min(floor(2^32 exp(-beta_t dE)), 2^32 - 2) with the C library's exponential.  An
+ * adaptive run keeps those of its current step only (PA_ERR_STATE for another). */
+int pa_get_thresholds(pa_ctx* ctx, int32_t t, uint32_t* out, int64_t cap);
 
 /* ---- instrumentation ----
  * Counters since the last pa_stats_reset: steps run, kernels launched by the
@@ -330,6 +336,17 @@ int pa_debug_lookback(pa_ctx* ctx, int32_t spins, int32_t withheld_tile);
  * couplings or an adaptive schedule, one_launch outside {0, 1}, withheld_block < -1,
  * or withheld_block >= 0 with one_launch = 0. */
 int pa_debug_bisect(pa_ctx* ctx, int32_t one_launch, int32_t withheld_block);
+
+/* ---- testing hook: the thresholds of a Gaussian-coupling run ----
+ * The device computes them and lists the few whose floor the last bits of the
+ * exponential decide; the host evaluates the listed ones.  This bounds the list to
+ * list_cap entries (-1: what its room holds), so that longer ones overflow (the tables
+ * are then built by halves, a single one by the host), and keeps the list out of pinned
+ * host memory with pinned = 0.  It applies to the later steps of an adaptive run; an
+ * explicit schedule's tables are built again at once.  The thresholds are the same
+ * whatever is set.  For tests only; PA_ERR_INVALID for a run without Gaussian couplings,
+ * list_cap < -1 or pinned outside {0, 1}. */
+int pa_debug_thresholds(pa_ctx* ctx, int32_t list_cap, int32_t pinned);
 
 /* Waits for the context's stream; returns the first recorded error, if any. */
 int pa_sync(pa_ctx* ctx);

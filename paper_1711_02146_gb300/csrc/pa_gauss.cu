@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kCountThreads) k_g_counts(RunGeom g, GArgs a, 
 // tables on eight host threads took 0.6 ms at L = 10, and all 60 tables of an L = 8
 // schedule, with a weight table for each, 45 of a run's 97 ms; the device idled.)
 __global__ void __launch_bounds__(256) k_g_site_tables(int L, const int32_t* __restrict__ Jq, double beta,
-                                                      uint32_t* gtab, int table, uint32_t* open) {
+                                                      uint32_t* gtab, int table, uint32_t* open, uint32_t cap) {
   const int e = blockIdx.x * 256 + threadIdx.x, N = L * L * L;
   if (e >= N * kGPatterns) return;
   const int n = e / kGPatterns, b = e % kGPatterns;
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(256) k_g_site_tables(int L, const int32_t* __r
     thr = (uint32_t)lo;
     if (lo != hi) {
       const uint32_t i = atomicAdd(&open[0], 1u);
-      if (i < (uint32_t)kGOpenCap) {
+      if (i < cap) {
         open[1 + 2 * i] = (uint32_t)table;
         open[2 + 2 * i] = (uint32_t)e;
       }
@@ -868,10 +868,10 @@ __global__ void __launch_bounds__(kLinkThreads) k_g_link(RunGeom g, GArgs a, int
 // ---------------------------------------------------------------- launchers
 
 int launch_g_site_tables(const RunGeom& g, const int32_t* Jq, double beta, uint32_t* gtab, int table, uint32_t* open,
-                         void* stream) {
+                         uint32_t cap, void* stream) {
   const int per = g.N * kGPatterns;
   k_g_site_tables<<<blocks_for(per, 256), 256, 0, (cudaStream_t)stream>>>(g.L, Jq, beta, gtab + (size_t)table * per,
-                                                                          table, open);
+                                                                          table, open, cap);
   return (int)cudaGetLastError();
 }
 

@@ -197,11 +197,13 @@ int launch_g_resample(const RunGeom& g, PopDev* pops, int cur, int t, const doub
 // each).  An entry whose floor could come out otherwise with another rounding of the
 // exponential (both this one and the C library's are within an ulp) is appended to the
 // list open = {length, entries}, two words per entry: its table, and site kGPatterns +
-// pattern; at most kGOpenCap entries are stored, the length counts all.
-constexpr int kGOpenCap = 127;
+// pattern; at most cap entries are stored, the length counts all.  Half of the 64 N
+// entries have dE > 0, and each is open with a chance of 2^-17 at most (an interval of
+// 2^-49 2^32 around an integer): N / 4096 entries per table, one at L = 16.
+constexpr int kGOpenCap = 127;  // of a single step's list
 constexpr int kGOpenWords = 1 + 2 * kGOpenCap;
 int launch_g_site_tables(const RunGeom& g, const int32_t* Jq, double beta, uint32_t* gtab, int table, uint32_t* open,
-                         void* stream);
+                         uint32_t cap, void* stream);
 int launch_g_sweep(const RunGeom& g, PopDev* pops, int cur, const uint32_t* jtab, const int32_t* Jq, long long Jtot,
                    const uint32_t* gtab, int t, int n_sweeps, void* stream);
 // Step 0: the energies of the initial population in spins[1], which moves to spins[0].

@@ -49,6 +49,9 @@ struct pa_ctx {
   double* wadapt = nullptr;     // adaptive schedule: the table of the current step
   double* wadapt_host = nullptr;  // its pinned host copy (uploaded without a wait)
   uint32_t* gopen_host = nullptr;  // pinned: the site-table entries the device leaves open, and their values
+  int32_t gopen_cap = -1;          // pa_debug_thresholds: entries that a list of them holds at most (-1: its room)
+  bool gopen_pageable = false;     // pa_debug_thresholds: no pinned memory for that list
+  int32_t gtab_step = -1;          // adaptive Gaussian schedule: the step whose tables gtab holds
   std::vector<int32_t> gw_slot;    // explicit Gaussian schedule: the weight table (in gw) of each step
   int32_t occ_span = -1;          // adaptive +-1: highest minus lowest occupied level of population 0
   // All device buffers of the run are carved from one stream-ordered allocation:
@@ -91,6 +94,7 @@ struct pa_ctx {
 namespace {
 
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? PA_OK : PA_ERR_CUDA; }
+int launch_rc(int e) { return e == 0 ? PA_OK : PA_ERR_CUDA; }
 
 // The step's sum over families of nu ln nu from its exact 128-bit fixed-point form
 // (units of 2^-100), rounded to double once.
@@ -393,16 +397,22 @@ uint32_t site_threshold(const std::vector<int32_t>& Jq, int L, double beta, int 
   return v > 4294967294.0 ? 0xFFFFFFFEu : (uint32_t)v;
 }
 
-// The device list of open entries, kept behind the sweep's tables in the scratch of
-// population 0's buffer buf (PopDev).
+// The device list of a step's open entries (adaptive schedule; kGOpenCap of them), kept
+// behind the sweep's tables in the scratch of population 0's buffer buf (PopDev).
 uint32_t* open_entries(const pa_ctx* c, int buf) {
   const RunGeom& g = c->g;
   return c->pops[0].spins[buf] + (size_t)g.pitch * g.sw + (size_t)g.N * pa::kGPatterns +
          (size_t)g.N / 2 * pa::kGPatterns;
 }
 
+// Entries that a list with room for `room` of them takes.
+uint32_t open_cap(const pa_ctx* c, size_t room) {
+  return (uint32_t)(c->gopen_cap >= 0 ? std::min((size_t)c->gopen_cap, room) : room);
+}
+
 // Pinned host memory for that list and for the entries' values (null where none is had).
 uint32_t* pinned_entries(pa_ctx* c) {
+  if (c->gopen_pageable) return nullptr;
   if (!c->gopen_host) {
     void* h = nullptr;
     if (cudaMallocHost(&h, sizeof(uint32_t) * (pa::kGOpenWords + pa::kGOpenCap)) == cudaSuccess)
@@ -413,25 +423,58 @@ uint32_t* pinned_entries(pa_ctx* c) {
   return c->gopen_host;
 }
 
-// Evaluates the listed entries (list[0] of them) of the tables of betas[first], betas[first
-// + 1], ... on the host and sends them to gtab, stream-ordered; values: kGOpenCap words
-// that stay alive until then.  A list that overflowed sends whole tables.
-int close_entries(pa_ctx* c, const uint32_t* list, uint32_t* values, const double* betas, size_t n_tables) {
+// Table `table` of gtab, for beta, from the host.
+int host_site_table(pa_ctx* c, size_t table, double beta) {
+  const size_t per = (size_t)c->g.N * pa::kGPatterns;
+  std::vector<uint32_t> tab(per);
+  for (size_t e = 0; e < per; ++e)
+    tab[e] = site_threshold(c->Jq_host, c->g.L, beta, (int)(e / pa::kGPatterns), (int)(e % pa::kGPatterns));
+  return copy_h2d(c, c->gtab + table * per, tab.data(), sizeof(uint32_t) * per);
+}
+
+// Evaluates the listed entries (list[0] of them) of the tables of betas[0], betas[1], ...
+// on the host and sends them to gtab, stream-ordered; values: a word for each that stays
+// alive until then.
+int close_entries(pa_ctx* c, const uint32_t* list, uint32_t* values, const double* betas) {
   const size_t per = (size_t)c->g.N * pa::kGPatterns;
   int rc = PA_OK;
-  if (list[0] > (uint32_t)pa::kGOpenCap) {
-    std::vector<uint32_t> tab(per);
-    for (size_t k = 0; k < n_tables && rc == PA_OK; ++k) {
-      for (size_t e = 0; e < per; ++e)
-        tab[e] = site_threshold(c->Jq_host, c->g.L, betas[k], (int)(e / pa::kGPatterns), (int)(e % pa::kGPatterns));
-      rc = copy_h2d(c, c->gtab + k * per, tab.data(), sizeof(uint32_t) * per);
-    }
-    return rc;
-  }
   for (uint32_t i = 0; i < list[0] && rc == PA_OK; ++i) {
     const size_t k = list[1 + 2 * i], e = list[2 + 2 * i];
     values[i] = site_threshold(c->Jq_host, c->g.L, betas[k], (int)(e / pa::kGPatterns), (int)(e % pa::kGPatterns));
     rc = copy_async(c, c->gtab + k * per + e, values + i, sizeof(uint32_t));
+  }
+  return rc;
+}
+
+// The tables of the steps [first, first + n) of an explicit schedule.  Their list takes
+// the room of table 0 (step 0 does not sweep): 32 N entries, what 131 072 tables leave open
+// on average.  Of a list that overflows only the length is of use; the tables are then
+// built again by halves, and one whose own list overflows comes from the host.
+int build_site_tables(pa_ctx* c, size_t first, size_t n) {
+  const size_t per = (size_t)c->g.N * pa::kGPatterns;
+  uint32_t* open = c->gtab;
+  const uint32_t cap = open_cap(c, (per - 1) / 2);
+  int rc = cuda_status(cudaMemsetAsync(open, 0, sizeof(uint32_t), c->stream));
+  for (size_t t = first; t < first + n && rc == PA_OK; ++t)
+    rc = launch_rc(pa::launch_g_site_tables(c->g, c->Jq, c->betas[t], c->gtab, (int)t, open, cap, c->stream));
+  std::vector<uint32_t> list(pa::kGOpenWords, 0u);
+  if (rc == PA_OK) rc = copy_d2h(c, list.data(), open, sizeof(uint32_t) * list.size());
+  if (rc != PA_OK) return rc;
+  if (list[0] > cap) {
+    if (n == 1) return host_site_table(c, first, c->betas[first]);
+    rc = build_site_tables(c, first, n / 2);
+    return rc == PA_OK ? build_site_tables(c, first + n / 2, n - n / 2) : rc;
+  }
+  if (list[0] > (uint32_t)pa::kGOpenCap) {  // the entries beyond the first copy
+    list.resize(1 + 2 * (size_t)list[0]);
+    rc = copy_d2h(c, list.data() + pa::kGOpenWords, open + pa::kGOpenWords,
+                  sizeof(uint32_t) * (list.size() - (size_t)pa::kGOpenWords));
+  }
+  std::vector<uint32_t> values(list[0]);
+  if (rc == PA_OK) rc = close_entries(c, list.data(), values.data(), c->betas.data());
+  if (list[0]) {  // values leaves scope
+    const int done = cuda_status(cudaStreamSynchronize(c->stream));
+    rc = rc == PA_OK ? done : rc;
   }
   return rc;
 }
@@ -636,8 +679,6 @@ void pm1_observables(const RunGeom& g, const std::vector<double>& betas, const S
   }
   *out = o;
 }
-
-int launch_rc(int e) { return e == 0 ? PA_OK : PA_ERR_CUDA; }
 
 // Adaptive step with Gaussian couplings (§IV.B), as for +-1 couplings: the largest
 // dbeta in (0, beta_max - beta] whose culling fraction (population 0, the
@@ -1202,14 +1243,7 @@ int create_run_impl(const pa_config* cfg, void* cuda_stream, pa_ctx** out, bool 
         for (size_t i = 0; i < d.size(); ++i)
           if (bits_of(d[i]) == bits_of(c->betas[t] - c->betas[t - 1])) c->gw_slot[t] = (int32_t)i;
       if (rc == PA_OK) rc = copy_async(c, c->gw, gw_all.data(), sizeof(double) * gw_all.size());
-      uint32_t* open = open_entries(c, 0);
-      std::vector<uint32_t> list(pa::kGOpenWords, 0u), values(pa::kGOpenCap);
-      if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(open, 0, sizeof(uint32_t), s));
-      for (size_t t = 1; t < T && rc == PA_OK; ++t)
-        rc = launch_rc(pa::launch_g_site_tables(g, c->Jq, c->betas[t], c->gtab, (int)t, open, s));
-      if (rc == PA_OK) rc = copy_d2h(c, list.data(), open, sizeof(uint32_t) * list.size());
-      if (rc == PA_OK) rc = close_entries(c, list.data(), values.data(), c->betas.data(), T);
-      if (rc == PA_OK && list[0]) rc = cuda_status(cudaStreamSynchronize(s));  // values leaves scope
+      if (rc == PA_OK) rc = build_site_tables(c, 1, T - 1);
     }
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->J, 0, (size_t)3 * g.N, s));
     if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(c->jtab, 0, sizeof(uint32_t) * 4 * g.N, s));
@@ -1284,11 +1318,12 @@ int pa_step(pa_ctx* c) try {
     // fraction is the one the bisection accepted, and the site tables of the beta just
     // chosen; the host settles the entries that the device left open while it resamples.
     uint32_t* open = open_entries(c, 1 - c->cur);
+    const uint32_t open_max = open_cap(c, pa::kGOpenCap);
     uint32_t* host = c->adaptive ? pinned_entries(c) : nullptr;
     if (c->adaptive) {
       if (rc == PA_OK) rc = launch_rc(pa::launch_g_tables(nullptr, dbeta, c->gw, c->stream));
       if (rc == PA_OK) rc = cuda_status(cudaMemsetAsync(open, 0, sizeof(uint32_t), s));
-      if (rc == PA_OK) rc = launch_rc(pa::launch_g_site_tables(c->g, c->Jq, c->betas[(size_t)t], c->gtab, 0, open, s));
+      if (rc == PA_OK) rc = launch_rc(pa::launch_g_site_tables(c->g, c->Jq, c->betas[(size_t)t], c->gtab, 0, open, open_max, s));
       if (host && rc == PA_OK) {
         c->stats.d2h_bytes += (int64_t)sizeof(uint32_t) * pa::kGOpenWords;
         rc = cuda_status(cudaMemcpyAsync(host, open, sizeof(uint32_t) * pa::kGOpenWords, cudaMemcpyDeviceToHost, s));
@@ -1303,15 +1338,14 @@ int pa_step(pa_ctx* c) try {
     }
     if (c->adaptive && rc == PA_OK) {
       const double beta = c->betas[(size_t)t];
-      if (host) {
-        rc = cuda_status(cudaEventSynchronize(c->gopen_ev));
-        if (rc == PA_OK) rc = close_entries(c, host, host + pa::kGOpenWords, &beta, 1);
-      } else {
-        std::vector<uint32_t> list(pa::kGOpenWords, 0u), values(pa::kGOpenCap);
-        rc = copy_d2h(c, list.data(), open, sizeof(uint32_t) * list.size());
-        if (rc == PA_OK) rc = close_entries(c, list.data(), values.data(), &beta, 1);
-        if (rc == PA_OK && list[0]) rc = cuda_status(cudaStreamSynchronize(s));  // values leaves scope
-      }
+      std::vector<uint32_t> pageable(host ? 0 : pa::kGOpenWords + pa::kGOpenCap, 0u);  // the list and its values
+      uint32_t* list = host ? host : pageable.data();
+      rc = host ? cuda_status(cudaEventSynchronize(c->gopen_ev))
+                : copy_d2h(c, list, open, sizeof(uint32_t) * pa::kGOpenWords);
+      if (rc == PA_OK)
+        rc = list[0] > open_max ? host_site_table(c, 0, beta) : close_entries(c, list, list + pa::kGOpenWords, &beta);
+      if (rc == PA_OK && !host && list[0]) rc = cuda_status(cudaStreamSynchronize(s));  // pageable leaves scope
+      c->gtab_step = rc == PA_OK ? t : -1;
     }
     if (rc == PA_OK) {
       PhaseTimer pt(c, PA_PHASE_SWEEP, 1 + c->g.n_pop);
@@ -1369,6 +1403,28 @@ int pa_debug_bisect(pa_ctx* c, int32_t one_launch, int32_t withheld_block) try {
   c->gbis_blocks = one_launch ? -1 : 0;  // -1: sized again at the next step
   c->gbis_withheld = withheld_block;
   return PA_OK;
+} catch (...) {
+  return pa::exception_status();
+}
+
+int pa_debug_thresholds(pa_ctx* c, int32_t list_cap, int32_t pinned) try {
+  if (!c || c->model != PA_MODEL_GAUSS || list_cap < -1 || pinned < 0 || pinned > 1) return PA_ERR_INVALID;
+  c->gopen_cap = list_cap;
+  c->gopen_pageable = !pinned;
+  const size_t T = c->betas.size();
+  return c->adaptive || T < 2 ? PA_OK : fail(c, build_site_tables(c, 1, T - 1));
+} catch (...) {
+  return pa::exception_status();
+}
+
+int pa_get_thresholds(pa_ctx* c, int32_t t, uint32_t* out, int64_t cap) try {
+  if (!c || !out || c->model != PA_MODEL_GAUSS || t < 1 || t >= c->cfg.n_temps) return PA_ERR_INVALID;
+  if (c->adaptive && t != c->gtab_step) return PA_ERR_STATE;
+  const size_t per = (size_t)c->g.N * pa::kGPatterns;
+  if (cap < (int64_t)per) return PA_ERR_CAPACITY;
+  const int rc = pa_sync(c);
+  return rc == PA_OK ? fail(c, copy_d2h(c, out, c->gtab + (c->adaptive ? 0 : (size_t)t) * per, sizeof(uint32_t) * per))
+                     : rc;
 } catch (...) {
   return pa::exception_status();
 }
