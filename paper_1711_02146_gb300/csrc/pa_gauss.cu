@@ -38,16 +38,15 @@ __host__ __device__ inline int blocks_for(long long n, int per) { return (int)((
 // the last that a 32-bit read at any site's z neighbour touches.
 __host__ __device__ inline int link_row_words(int N, int L) { return (N + 31 + L * L) / 32 + 2; }
 
-// Opens the records of step t (what k_g_weights does for t >= 1).
-__global__ void k_g_open(GArgs a, int t) {
-  GRec& r = a.p[threadIdx.x].grec[t];
+// Opens a step's record: all of it, since a checkpoint saves the bytes.
+__device__ __forceinline__ void open_record(GRec& out) {
+  GRec r{};
   r.E_min = 0x7fffffffffffffffLL;
-  r.E0 = 0;
-  r.sum_E = 0;
-  r.sum_E2_lo = r.sum_E2_hi = 0;
-  r.n_at_E0 = 0;
-  r.ql_sum = 0;
+  out = r;
 }
+
+// The records of step t (k_g_weights opens those of t >= 1).
+__global__ void k_g_open(GArgs a, int t) { open_record(a.p[threadIdx.x].grec[t]); }
 
 // ---------------------------------------------------------------- resampling
 
@@ -159,13 +158,7 @@ __global__ void __launch_bounds__(kChunk) k_g_weights(RunGeom g, GArgs a, int t,
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     P.rec[t].R_prev = R_old;
-    GRec& r = P.grec[t];
-    r.E_min = 0x7fffffffffffffffLL;
-    r.E0 = 0;
-    r.sum_E = 0;
-    r.sum_E2_lo = r.sum_E2_hi = 0;
-    r.n_at_E0 = 0;
-    r.ql_sum = 0;
+    open_record(P.grec[t]);
   }
 }
 
