@@ -235,14 +235,20 @@ int copy_h2d(pa_ctx* c, void* dst, const void* src, size_t bytes) {
 // of n rounded up to 32 bytes: a spin buffer that holds nothing of use).
 int64_t row_bytes(int64_t n) { return (n + 31) / 32 * 32; }
 
+int unpack_rows(pa_ctx* c, const uint32_t* spins, int64_t first, int64_t n, int8_t* scratch) {
+  return launch_rc(pa::launch_unpack_rows(c->g, spins, first, n, row_bytes(n), scratch, c->stream));
+}
+
+// What unpack_rows left in scratch, stream-ordered.
+int copy_unpacked(pa_ctx* c, int64_t n, const int8_t* scratch, void* host) {
+  c->stats.d2h_bytes += (int64_t)c->g.N * n;
+  return cuda_status(cudaMemcpy2DAsync(host, (size_t)n, scratch, (size_t)row_bytes(n), (size_t)n, (size_t)c->g.N,
+                                       cudaMemcpyDeviceToHost, c->stream));
+}
+
 int copy_rows_d2h(pa_ctx* c, const uint32_t* spins, int64_t first, int64_t n, int8_t* scratch, void* host) {
-  const RunGeom& g = c->g;
-  const size_t ld = (size_t)row_bytes(n);
-  int rc = pa::launch_unpack_rows(g, spins, first, n, (int64_t)ld, scratch, c->stream) == 0 ? PA_OK : PA_ERR_CUDA;
-  c->stats.d2h_bytes += (int64_t)g.N * n;
-  if (rc == PA_OK)
-    rc = cuda_status(cudaMemcpy2DAsync(host, (size_t)n, scratch, ld, (size_t)n, (size_t)g.N, cudaMemcpyDeviceToHost,
-                                       c->stream));
+  int rc = unpack_rows(c, spins, first, n, scratch);
+  if (rc == PA_OK) rc = copy_unpacked(c, n, scratch, host);
   return rc == PA_OK ? cuda_status(cudaStreamSynchronize(c->stream)) : rc;
 }
 
@@ -254,6 +260,19 @@ int copy_rows_h2d(pa_ctx* c, uint32_t* spins, int64_t n, int8_t* scratch, const 
                                          c->stream));
   if (rc == PA_OK) rc = pa::launch_pack_rows(g, scratch, n, (int64_t)ld, spins, c->stream) == 0 ? PA_OK : PA_ERR_CUDA;
   return rc == PA_OK ? cuda_status(cudaStreamSynchronize(c->stream)) : rc;
+}
+
+// n rows of bits as int8 spins [n][N], eight sites (a byte of a row) at a time: with each
+// byte of m holding its own bit of x, the sum carries into a byte's top bit where it is set.
+void expand_rows(const uint32_t* rows, int sw, int N, int64_t n, int8_t* out) {
+  for (int64_t j = 0; j < n; ++j)
+    for (int k = 0; k < N / 8; ++k) {
+      const uint64_t x = rows[j * sw + k / 4] >> (8 * (k % 4)) & 0xFFu;
+      const uint64_t m = (x * 0x0101010101010101ull) & 0x8040201008040201ull;
+      const uint64_t set = ((m + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
+      const uint64_t spins = set * 0xFEu + 0x0101010101010101ull;
+      std::memcpy(out + (size_t)j * N + 8 * (size_t)k, &spins, 8);
+    }
 }
 
 // Stream-ordered host-to-device copy; the caller keeps src alive until the stream
@@ -1597,6 +1616,11 @@ int pa_population_size(pa_ctx* c, int32_t pop, int64_t* count) try {
   return pa::exception_status();
 }
 
+// Spins up to which a read-out copies rows of bits and expands them here, beyond which the
+// device expands them: a launch before the copy takes 10 us (one replica of L = 4: 83 us
+// against 73), the host 2.4 ns for eight spins (16 of L = 16, 65536: 84 us against 94).
+constexpr int64_t kExpandOnHost = 1 << 14;
+
 int pa_get_replicas(pa_ctx* c, int32_t pop, int64_t first, int64_t n, int8_t* spins, int32_t* labels,
                     int32_t* energies) try {
   if (!c || pop < 0 || pop >= c->g.n_pop || first < 0 || n < 0) return PA_ERR_INVALID;
@@ -1607,7 +1631,12 @@ int pa_get_replicas(pa_ctx* c, int32_t pop, int64_t first, int64_t n, int8_t* sp
   if (n == 0) return PA_OK;
   const RunGeom& g = c->g;
   const PopDev& P = c->pops[pop];
-  if (spins) {
+  if (spins && n * g.N <= kExpandOnHost) {
+    std::vector<uint32_t> rows((size_t)n * g.sw);
+    rc = copy_d2h(c, rows.data(), P.spins[c->cur] + first * g.sw, sizeof(uint32_t) * rows.size());
+    if (rc != PA_OK) return fail(c, rc);
+    expand_rows(rows.data(), g.sw, g.N, n, spins);
+  } else if (spins) {
     // expanded on the device into the buffer that does not hold the population
     int8_t* out = reinterpret_cast<int8_t*>(P.spins[1 - c->cur]);
     rc = launch_rc(pa::launch_unpack_replicas(g, P.spins[c->cur], first, n, out, c->stream));
@@ -1836,21 +1865,26 @@ int pa_checkpoint(pa_ctx* c, void* buf, size_t cap, size_t* size) try {
   o += sizeof(double) * (size_t)c->cfg.n_temps;
   std::memcpy(o, c->sweeps.data(), sizeof(int32_t) * (size_t)c->cfg.n_temps);
   o += sizeof(int32_t) * (size_t)c->cfg.n_temps;
+  // The spins are expanded while the first copies run, and one wait serves all copies.
+  for (int p = 0; p < g.n_pop && rc == PA_OK; ++p)
+    if (Rt[p])
+      rc = unpack_rows(c, c->pops[p].spins[c->cur], 0, Rt[p], reinterpret_cast<int8_t*>(c->pops[p].spins[1 - c->cur]));
+  auto get = [&](const void* src, size_t bytes) {
+    if (rc == PA_OK && bytes) {
+      c->stats.d2h_bytes += (int64_t)bytes;
+      rc = cuda_status(cudaMemcpyAsync(o, src, bytes, cudaMemcpyDeviceToHost, c->stream));
+    }
+    o += bytes;
+  };
   for (int p = 0; p < g.n_pop && rc == PA_OK; ++p) {
     const PopDev& P = c->pops[p];
     const size_t R = (size_t)Rt[p];
-    auto get = [&](const void* src, size_t bytes) {
-      if (rc == PA_OK && bytes) rc = copy_d2h(c, o, src, bytes);
-      o += bytes;
-    };
     get(P.rec, sizeof(StepRec) * (size_t)(t + 1));
     if (gauss)
       get(P.grec, sizeof(pa::GRec) * (size_t)(t + 1));
     else
       get(P.hist, sizeof(uint32_t) * (size_t)(t + 1) * (size_t)g.n_levels);
-    if (rc == PA_OK && R) {
-      rc = copy_rows_d2h(c, P.spins[c->cur], 0, (int64_t)R, reinterpret_cast<int8_t*>(P.spins[1 - c->cur]), o);
-    }
+    if (rc == PA_OK && R) rc = copy_unpacked(c, (int64_t)R, reinterpret_cast<int8_t*>(P.spins[1 - c->cur]), o);
     o += (size_t)g.N * R;
     get(P.labels[c->cur], sizeof(int32_t) * R);
     if (gauss)
@@ -1863,8 +1897,10 @@ int pa_checkpoint(pa_ctx* c, void* buf, size_t cap, size_t* size) try {
     get(P.mhist, sizeof(int32_t) * (R + 1));
   }
   const size_t qbytes = sizeof(unsigned long long) * (size_t)(t + 1) * (size_t)g.q_bins;
-  if (rc == PA_OK) rc = copy_d2h(c, o, c->qhist, qbytes);
-  if (rc == PA_OK && gauss) rc = copy_d2h(c, o + qbytes, c->qlhist, qbytes);
+  get(c->qhist, qbytes);
+  if (gauss) get(c->qlhist, qbytes);
+  const int done = cuda_status(cudaStreamSynchronize(c->stream));
+  rc = rc == PA_OK ? done : rc;
   return rc == PA_OK ? PA_OK : fail(c, rc);
 } catch (...) {
   return pa::exception_status();

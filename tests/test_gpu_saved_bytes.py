@@ -28,3 +28,23 @@ def test_gaussian_checkpoint_holds_no_stale_memory(pa):
         saved.append(run.checkpoint())
         run.close()
     assert saved[0] == saved[1]
+
+
+@pytest.mark.parametrize("L,R", [(2, 3000), (6, 200), (10, 60), (16, 30)])
+@pytest.mark.parametrize("model", [0, 1])
+def test_few_replicas_equal_the_population(pa, L, R, model):
+    """Read-outs of up to 16384 spins cross the link as rows of bits, larger ones as bytes."""
+    run = pa.Run(L, R, 3, 4, np.linspace(0.0, 0.4, 3), n_sweeps=1, model=model)
+    run.run()
+    spins, labels, _ = run.population()
+    N, most = L ** 3, 16384 // L ** 3
+    assert len(spins) > most + 4
+    out, lab = np.zeros((most + 1, N), dtype=np.int8), np.zeros(most + 1, dtype=np.int32)
+    for n in (1, 3, most, most + 1):  # most is 4 at the least
+        run.stats_reset()
+        rc = pa.lib().pa_get_replicas(run._h, 0, 3, n, pa._p(out, pa.ctypes.c_int8), pa._p(lab, pa.ctypes.c_int32), None)
+        assert rc == pa.PA_OK
+        assert np.array_equal(out[:n], spins[3:3 + n]) and np.array_equal(lab[:n], labels[3:3 + n])
+        row = 4 * ((N + 31) // 32) if N <= 64 else 32 * ((N + 255) // 256)
+        assert run.stats()["d2h_bytes"] - 4 * n - 8 == (n * row if n <= most else n * N)  # labels; size and status
+    run.close()
