@@ -524,9 +524,8 @@ int pa_sweep_autotune(int32_t L, int32_t R, int32_t launches, double* ms_per_lau
  * is written as 0, *n_new is set to -1 and no parent is written.  Nothing is
  * ever written outside counts[0, n_old) and parents[0, parents_cap).
  *
- * It allocates nothing: its scratch (the per-block totals and offsets of the
- * scan and an error mark) is a fixed array of 4097 64-bit words (about 32 KiB)
- * in the library's device memory, held by every GPU that loads the library
+ * It allocates nothing: its scratch (the copy totals of the blocks of 1024
+ * slots) is a fixed array of 4096 64-bit words (32 KiB) in the library's device memory, held by every GPU that loads the library
  * until the process exits, which limits n_old to PA_NOALLOC_MAX_SLOTS (larger
  * inputs return PA_ERR_INVALID before any launch).  All calls on a device share
  * that array: calls whose work overlaps on the GPU (other streams, other host

@@ -31,7 +31,7 @@ constexpr int kNaMaxDevices = 64;
 
 // [0, n_blocks): block totals (64-bit: a block of 1024 slots may hold up to 2^41
 // copies); a block whose inputs are invalid writes -1 as its total.
-__device__ __align__(256) long long g_na_scratch[PA_NOALLOC_MAX_BLOCKS + 1];
+__device__ __align__(256) long long g_na_scratch[PA_NOALLOC_MAX_BLOCKS];
 
 __device__ __forceinline__ long long warp_inclusive_scan_ll(long long v) {
   const int lane = threadIdx.x & 31;
@@ -110,11 +110,22 @@ __global__ void __launch_bounds__(kNaThreads) k_na_counts(const int32_t* __restr
 }
 
 // Parents of the new slots j < cap: slot offset_i + q (q < n_i) descends from old
-// slot i.  Every block reads all block totals: those before it give its offset, and a
-// negative one anywhere means invalid input, for which nothing is written but *n_new = -1;
-// the last block writes the grand total, the new population size.  (A scan kernel of one
-// block in between cost 1.9 us and a launch: 18.4 us per call at 1e6 slots against 12.)
+// slot i.  A block takes the slots of PER counting blocks.  It reads all block totals: those
+// before its own give its offset, and a negative one anywhere means invalid input, for which
+// nothing is written but *n_new = -1; the last block writes the grand total, the new
+// population size.  (A scan kernel of one block in between cost 1.9 us and a launch: 18.5 us
+// per call at 1e6 slots against 14.6.)  The totals are read blocks x totals times: with
+// PER = 1 the 4096 blocks of the largest population read 134 MB of them, 39.0 us per call at
+// 4 194 304 slots where the scan kernel's form took 37.3; PER = 2 takes 36.8, and 24.7 at
+// 2.5e6 (26.0).  PER = 2 from 1 048 577 slots on is slower there (16.5 us against 14.5: half
+// the chip's places stay empty), eight slots in a row per thread at 4 194 304 (38.9: four
+// times the lines per store), and the counts of both blocks loaded ahead as slow as PER = 1.
+// With PER = 1 a thread loads its counts before the scan of the totals, and the total is
+// written before the parents (15.0 us at 1e6 slots otherwise, 14.5 so).
 // The launch overlaps the counting kernel's end; griddepcontrol.wait orders the reads.
+constexpr int kNaScatterBlocks = 2048;  // PER = 1 up to these many, 2 beyond
+
+template <int PER>
 __global__ void __launch_bounds__(kNaThreads) k_na_scatter(const int32_t* __restrict__ counts, int n_old, int n_blocks,
                                                            const long long* __restrict__ scratch, int32_t* parents,
                                                            long long cap, int64_t* n_new) {
@@ -125,25 +136,33 @@ __global__ void __launch_bounds__(kNaThreads) k_na_scatter(const int32_t* __rest
   for (int b = threadIdx.x; b < n_blocks; b += kNaThreads) {
     const long long v = __ldcg(scratch + b);
     bad |= v < 0;
-    if (b < (int)blockIdx.x) before += v;
+    if (b < PER * (int)blockIdx.x) before += v;
   }
   bad = __syncthreads_or(bad);
-  const int i0 = blockIdx.x * kNaSlotsPerBlock + 4 * threadIdx.x;
-  long long n[4] = {0, 0, 0, 0};
+  long long n[4], base, mine;
+  auto load = [&](int i0) {
 #pragma unroll
-  for (int b = 0; b < 4; ++b)
-    if (!bad && i0 + b < n_old) n[b] = __ldcg(counts + i0 + b);
-  long long base, mine;
+    for (int b = 0; b < 4; ++b) n[b] = !bad && i0 + b < n_old ? __ldcg(counts + i0 + b) : 0;
+  };
+  if (PER == 1) load(blockIdx.x * kNaSlotsPerBlock + 4 * threadIdx.x);
   block_exclusive_scan_ll(before, sh, &base);
-  long long off = base + block_exclusive_scan_ll(n[0] + n[1] + n[2] + n[3], sh, &mine);
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_new = bad ? -1 : base + mine;
-  if (bad) return;
+  const int first = PER * blockIdx.x, last = min(first + PER, n_blocks);
+  for (int blk = first; blk == first || blk < last; ++blk) {  // the slots of one counting block after the other
+    const int i0 = blk * kNaSlotsPerBlock + 4 * threadIdx.x;
+    if (PER > 1) load(i0);
+    long long off = base + block_exclusive_scan_ll(n[0] + n[1] + n[2] + n[3], sh, &mine);
+    base += mine;
+    if (PER == 1 && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_new = bad ? -1 : base;
+    if (PER == 1 && bad) return;
 #pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    for (long long j = off; j < off + n[b] && j < cap; ++j)
-      if (j >= 0) parents[j] = i0 + b;
-    off += n[b];
+    for (int b = 0; b < 4; ++b) {
+      for (long long j = off; j < off + n[b] && j < cap; ++j)
+        if (j >= 0) parents[j] = i0 + b;
+      off += n[b];
+    }
+    if (PER == 1) return;
   }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *n_new = bad ? -1 : base;
 }
 
 std::mutex g_na_mutex;
@@ -185,7 +204,8 @@ extern "C" int pa_resample_counts_noalloc(const int32_t* levels, int64_t n_old, 
   if (n_blocks > 0)
     k_na_counts<<<n_blocks, kNaThreads, 0, s>>>(levels, (int)n_old, fl, thr, n_levels, k0, k1, t, counts, scratch);
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)std::max(n_blocks, 1));  // an empty population: one block writes the total
+  const int per = n_blocks > kNaScatterBlocks ? 2 : 1;
+  cfg.gridDim = dim3((unsigned)std::max((n_blocks + per - 1) / per, 1));  // an empty population: one block writes the total
   cfg.blockDim = dim3(kNaThreads);
   cfg.stream = s;
   cudaLaunchAttribute overlap{};
@@ -193,8 +213,9 @@ extern "C" int pa_resample_counts_noalloc(const int32_t* levels, int64_t n_old, 
   overlap.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &overlap;
   cfg.numAttrs = n_blocks > 0 ? 1u : 0u;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_na_scatter, (const int32_t*)counts, (int)n_old, n_blocks,
-                                           (const long long*)scratch, parents, (long long)parents_cap, n_new);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, per == 2 ? k_na_scatter<2> : k_na_scatter<1>, (const int32_t*)counts,
+                                           (int)n_old, n_blocks, (const long long*)scratch, parents,
+                                           (long long)parents_cap, n_new);
   if (e != cudaSuccess) return PA_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? PA_OK : PA_ERR_CUDA;
 }
