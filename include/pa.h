@@ -337,6 +337,12 @@ int pa_debug_lookback(pa_ctx* ctx, int32_t spins, int32_t withheld_tile);
  * or withheld_block >= 0 with one_launch = 0. */
 int pa_debug_bisect(pa_ctx* ctx, int32_t one_launch, int32_t withheld_block);
 
+/* Bounds the blocks of the one-launch form for the later steps (0: as many as the
+ * population and the device take), so that a small population reaches what only a large
+ * one does otherwise: each warp's second chunk of replicas, and those beyond it.  The
+ * results are the same.  For tests only; PA_ERR_INVALID as above, or for n_blocks < 0. */
+int pa_debug_bisect_blocks(pa_ctx* ctx, int32_t n_blocks);
+
 /* ---- testing hook: the thresholds of a Gaussian-coupling run ----
  * The device computes them and lists the few whose floor the last bits of the
  * exponential decide; the host evaluates the listed ones.  This bounds the list to

@@ -80,6 +80,7 @@ struct pa_ctx {
   unsigned long long* gbar = nullptr;    // device: that launch's grid barrier words
   int gbis_blocks = -1;                  // blocks of the one-launch bisection (0: launch per halving)
   int gbis_withheld = -1;                // pa_debug_bisect: block kept from the first barrier
+  int gbis_most = 0;                     // pa_debug_bisect_blocks: blocks of the one launch at most (0: no bound)
   std::vector<int32_t> Jq_host;
   pa::LookbackTest lookback;             // pa_debug_lookback (tests of the bounded wait)
   // Completion events of the last steps (a ring, step u in entry u & 3, -1: none), so
@@ -712,11 +713,11 @@ int choose_dbeta_gauss(pa_ctx* c, double* dbeta) {
   const double target = c->cfg.eps_target;
   double b[4] = {0.0, rem, rem, 0.0};
   if (c->gbis_blocks < 0) c->gbis_blocks = pa::g_bisect_blocks(c->g);
+  const int n_blocks = c->gbis_most > 0 ? std::min(c->gbis_most, c->gbis_blocks) : c->gbis_blocks;
   int rc;
-  if (c->gbis_blocks > 0) {
+  if (n_blocks > 0) {
     rc = launch_rc(pa::launch_g_bisect_fused(c->g, c->pops, t, c->gbt, c->gbt + 3 * (size_t)pa::kGTableWeights,
-                                             c->gbar, c->gbis, rem, target, 64, c->gbis_blocks, c->gbis_withheld,
-                                             c->stream));
+                                             c->gbar, c->gbis, rem, target, 64, n_blocks, c->gbis_withheld, c->stream));
     if (rc == PA_OK) rc = copy_d2h(c, b, c->gbis, sizeof b);
     if (rc != PA_OK) return rc;
     if (b[3] < 0.0) return PA_ERR_TIMEOUT;
@@ -1421,6 +1422,14 @@ int pa_debug_bisect(pa_ctx* c, int32_t one_launch, int32_t withheld_block) try {
     return PA_ERR_INVALID;
   c->gbis_blocks = one_launch ? -1 : 0;  // -1: sized again at the next step
   c->gbis_withheld = withheld_block;
+  return PA_OK;
+} catch (...) {
+  return pa::exception_status();
+}
+
+int pa_debug_bisect_blocks(pa_ctx* c, int32_t n_blocks) try {
+  if (!c || c->model != PA_MODEL_GAUSS || !c->adaptive || n_blocks < 0) return PA_ERR_INVALID;
+  c->gbis_most = n_blocks;
   return PA_OK;
 } catch (...) {
   return pa::exception_status();

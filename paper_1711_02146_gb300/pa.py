@@ -176,6 +176,7 @@ SIGNATURES = {
     "pa_stats_reset": (ctypes.c_int, [_vp, ctypes.c_int]),
     "pa_debug_lookback": (ctypes.c_int, [_vp, ctypes.c_int32, ctypes.c_int32]),
     "pa_debug_bisect": (ctypes.c_int, [_vp, ctypes.c_int32, ctypes.c_int32]),
+    "pa_debug_bisect_blocks": (ctypes.c_int, [_vp, ctypes.c_int32]),
     "pa_debug_thresholds": (ctypes.c_int, [_vp, ctypes.c_int32, ctypes.c_int32]),
     "pa_get_thresholds": (ctypes.c_int, [_vp, ctypes.c_int32, ctypes.POINTER(ctypes.c_uint32), ctypes.c_int64]),
     "pa_get_stats": (ctypes.c_int, [_vp, ctypes.POINTER(Stats)]),
