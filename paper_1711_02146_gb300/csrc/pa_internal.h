@@ -1,5 +1,5 @@
 // pa_internal.h — structures shared by the host runtime (pa_runtime.cpp) and
-// the kernels (pa_kernels.cu, pa_sweep.cu).  Plain C++ (no CUDA types) so the
+// the kernels (pa_kernels.cu, pa_gauss.cu, pa_sweep*).  Plain C++ (no CUDA types) so the
 // runtime can be compiled by the host compiler alone.
 #pragma once
 #include <cstddef>
@@ -151,7 +151,7 @@ void sweep_tail_plan(int L, int shape, int64_t R, int n_sm, int32_t* tail_shape,
 constexpr int kCountThreads = 256;     // threads per resampling block
 constexpr int kSlotsPerCountBlock = 1024;
 
-// ---- launchers (pa_kernels.cu / pa_sweep.cu); each returns a cudaError_t as int ----
+// ---- launchers (pa_kernels.cu, pa_gauss.cu, pa_sweep*.cu); each returns a cudaError_t as int ----
 int launch_init_couplings(const RunGeom& g, uint64_t disorder_seed, int8_t* J, uint32_t* jtab, void* stream);
 // The initial spins into spins[buf] and labels (slot numbers) into labels[1 - buf]: the
 // step-0 sweep launch (no sweeps, every slot its own parent) takes the spins from
@@ -189,7 +189,7 @@ int launch_families(const RunGeom& g, PopDev* pops, int cur, int t, void* stream
 // The family-size histogram m(eta) of population pop at step t into its mhist
 // (on request: the step records are not touched).
 int launch_family_hist(const RunGeom& g, PopDev* pops, int pop, int cur, int t, void* stream);
-// Gaussian-coupling model (pa_gauss.cu, and k_sweep_g in pa_sweep.cu)
+// Gaussian-coupling model (pa_gauss.cu, and k_sweep_g in pa_sweep_gauss.cu)
 int launch_scan_scatter(const RunGeom& g, PopDev* pops, int cur, int t, int32_t* status, void* stream);
 int launch_g_resample(const RunGeom& g, PopDev* pops, int cur, int t, const double* wtab, int32_t* status,
                       void* stream);

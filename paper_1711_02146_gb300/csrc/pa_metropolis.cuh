@@ -1,6 +1,6 @@
 // pa_metropolis.cuh — the bit-sliced Metropolis test of the +-1 sweeps (32 replicas
 // per word) and the Philox blocks behind it, shared by the shared-memory sweep
-// (pa_sweep.cu), its Gaussian counterpart (Philox only) and the sweep of large
+// (pa_sweep_tile.cuh), its Gaussian counterpart (Philox only) and the sweep of large
 // lattices in global memory (pa_sweep_global.cu).
 #pragma once
 #include <cstdint>
@@ -156,7 +156,7 @@ __device__ __forceinline__ void philox_block(uint32_t uc, const SiteRec& sr, con
   philox_block(uc, sr.ua, sr.ub, tp, k0, k1, w);
 }
 
-// The plane's threshold bit of each replica of a word (SweepArgs::tm), from bits
+// The plane's threshold bit of each replica of a word (MetropolisArgs::tm), from bits
 // u0, u1 of its unsatisfied-bond count.
 __device__ __forceinline__ uint32_t threshold_bits(const uint32_t* tm, uint32_t u0, uint32_t u1) {
   return tm[0] ^ (u0 & tm[1]) ^ (u1 & tm[2]);

@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(kNaThreads) k_na_counts(const int32_t* __restr
 // PER = 1 the 4096 blocks of the largest population read 134 MB of them, 39.0 us per call at
 // 4 194 304 slots where the scan kernel's form took 37.3; PER = 2 takes 36.8, and 24.7 at
 // 2.5e6 (26.0).  PER = 2 from 1 048 577 slots on is slower there (16.5 us against 14.5: half
-// the chip's places stay empty), eight slots in a row per thread at 4 194 304 (38.9: four
-// times the lines per store), and the counts of both blocks loaded ahead as slow as PER = 1.
+// the chip's places stay empty), and eight slots in a row per thread (up to 38.9 at
+// 4 194 304) and the counts of both blocks loaded ahead (39.0 at 4e6) are no faster than PER = 1.
 // With PER = 1 a thread loads its counts before the scan of the totals, and the total is
 // written before the parents (15.0 us at 1e6 slots otherwise, 14.5 so).
 // The launch overlaps the counting kernel's end; griddepcontrol.wait orders the reads.

@@ -9,7 +9,7 @@
 //
 // One bit per spin keeps the words of moderate populations in the L2 cache (35 MB at
 // L = 24 and 2e4 replicas) for all half-sweeps of a step, so a half-sweep is bound by
-// integer issue, as the tile kernel is.  L = 24, R = 2e4, ten steps of ten sweeps: 17.8 ms
+// integer issue, as the tile kernel is.  L = 24, R = 2e4, ten steps of ten sweeps: 14.4 ms
 // for the whole run, from 328 ms with int8 spins (276 MB) and eight replicas per thread
 // decided one bit at a time (233 ms of half-sweeps, 90 ms of level counts).
 #include <cuda_runtime.h>
