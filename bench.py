@@ -58,6 +58,7 @@ UNIT = "updates/s"
 # 8 bytes of parent index and energy level per replica.
 
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "sweep_L10_R1e6_adaptive.txt")
+GAUSS_KERNEL = "k_sweep_g<10,8,128,4>"  # the Gaussian sweep at L = 10 has one launch shape
 GAUSS_PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "sweep_gauss_L10_R1e6_linear101.txt")
 SWEEP_SOURCES = [os.path.join(ROOT, "paper_1711_02146_gb300", "csrc", f) for f in
                  ("pa_bits.cuh", "pa_metropolis.cuh", "pa_sweep_tile.cuh", "pa_sweep_gauss.cu", "pa_sweep_l10.cu")]
@@ -338,6 +339,19 @@ def profile_traffic(kernel: str = "k_sweep<10,32,640,1>", tail=None):
         return None
 
 
+def step_traffic(kernel: str = "k_sweep<10,32,640,1>", tail=None):
+    """DRAM bytes of one step's sweep at R = 1e6 from the committed ncu summary, if it was
+    taken with the launch shapes in use (else None), and whether on the current source.  (A
+    bit per spin: 2 x 128 MB of rows, part of which stays in L2 from step to step.)"""
+    vals = profile_lines(PROFILE_SUMMARY)
+    if vals.get("sweep_kernel") != kernel or vals.get("sweep_tail_kernel", "none") != (tail or "none"):
+        return None, False
+    try:
+        return float(vals["dram_bytes_per_step"]), vals.get("sweep_source_sha256_16") == source_digest()
+    except (KeyError, ValueError):
+        return None, False
+
+
 def ops_per_update(path: str):
     """(instructions per update, instructions per clock per SM, their kind, whether they
     were profiled on the current source) from a committed profile summary."""
@@ -555,7 +569,7 @@ def gaussian_measurement(pa, steps: int, warmup: int, n_sm: int, cpu: bool, R: i
     out = {"workload": w.name, "steps_timed": f"temperature steps {warmup + 1}..{warmup + done}",
            "value": st["updates"] / (ms / 1e3), "unit": UNIT, "ms_per_step": ms / max(done, 1),
            "sweep": {"achieved": achieved, "peak": peak, "unit": "Gupdates/s", "frac": achieved / peak if peak else None,
-                     "peak_basis": peak_basis, "launch_ms": sweep_ms, "kernel": "k_sweep_g<10,32,640,1>"},
+                     "peak_basis": peak_basis, "launch_ms": sweep_ms, "kernel": GAUSS_KERNEL},
            "phase_share": {k: v / max(ms, 1e-9) for k, v in st["phase_ms"].items()},
            "last_step": {"beta": o["beta"], "R_tilde": o["R_tilde"], "mean_E_per_spin": o["mean_E"] / w.N,
                          "rho_t": o["rho_t"]}}
@@ -704,14 +718,16 @@ def ours(args):
     peak, peak_basis = issue_peak(n_sm, sm_mhz, PROFILE_SUMMARY)   # Gupdates/s
     achieved = updates_per_launch / (sweep_ms / 1e3) / 1e9
     kernel = f"k_sweep<{w.L},{shape['words']},{shape['threads']},{shape['ctas_per_sm']}>"
-    traffic = profile_traffic(kernel, tail_kernel(w.L, tail))
-    if traffic is not None:
-        traffic = traffic * updates_per_launch / (w.n_sweeps * w.N * w.R)
     replicas = updates_per_launch / (w.n_sweeps * w.N)
+    traffic, traffic_current = step_traffic(kernel, tail_kernel(w.L, tail))
+    if traffic is not None:
+        traffic *= replicas / 1e6
     hbm_bytes = 2.0 * w.N / 8.0 * replicas + 8.0 * replicas
     hbm_peak = measured_hbm_gbs()
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gupdates/s",
                 "frac": achieved / peak if peak else None, "traffic": traffic,
+                "traffic_basis": None if traffic is None else "DRAM bytes of a step's sweep (ncu, R = 1e6, "
+                                 f"{'this source' if traffic_current else 'an earlier source of the kernel'})",
                 "kernel": kernel if tail is None else f"{kernel} + {tail_kernel(w.L, tail)} from slot "
                                                       f"{plan['tail_from']}",
                 "launch_ms": sweep_ms, "updates_per_launch": updates_per_launch,
@@ -738,7 +754,7 @@ def ours(args):
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": done,
             "warmup": args.warmup, "ms_per_step": ms / max(done, 1), "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "int8", "data": "synthetic",
+            "scaling": "weak", "vs_baseline": None, "dtype": "bit", "data": "synthetic",
             "config": {"workload": w.name, "L": w.L, "R": w.R, "eps_target": w.eps_target, "beta_max": w.beta_max,
                        "n_sweeps": w.n_sweeps, "steps_timed": f"temperature steps {args.warmup + 1}.."
                                                               f"{args.warmup + done}",
