@@ -68,7 +68,7 @@ extern "C" {
  * q_bins       overlap histogram bins over q in [-1, 1] (odd, >= 3; 65 typical).
  * model        PA_MODEL_PM1: couplings +-1 with p = 1/2; PA_MODEL_GAUSS: couplings
  *              ~ N(0,1) (the paper's model, §II.A), clamped to [-5, 5] and held in
- *              fixed point (units of 2^-20), explicit schedules only.
+ *              fixed point (units of 2^-20).
  * The configuration and the arrays it points to are copied by pa_create. */
 #define PA_MODEL_PM1 0
 #define PA_MODEL_GAUSS 1
